@@ -826,54 +826,69 @@ __global__ void __launch_bounds__(NTHREADS, 2)
 // ---------------------------------------------------------------------------
 // histogram adjoint over per-bin rows (at most RB bins, non-degenerate
 // centres): the forward's row tables and walkers (device.cuh), built here
-// from the parameters, mirrored for the maximum as above.  Per piece all
-// factors are linear; the own product (degree 4), each leave-one-out product
-// LOO_n (degree 3) and LOO_n times the in-bin weight (e_{k+1} - x) / h_n
-// (degree 4) are integrated exactly by the 3-point Gauss-Legendre rule at
-// shared nodes, the leave-one-out products from pair products.  Every lane
-// runs the same steps; row reads at crossings are predicated, partials are
-// stored when a neighbour leaves a bin (or the centre leaves one of its own).
+// from the parameters, mirrored for the maximum as above.  On a piece every
+// factor is linear, f_i = m_i - D_i t for t in [-1, 1] (m_i its middle value,
+// D_i half its fall), so with the mean of t^2 = 1/3 and of t^4 = 1/5 every
+// integral is a short sum of products of non-negative numbers:
+//   f_0 f_1 = p - b t + e t^2, p = m_0 m_1, e = D_0 D_1, b = m_0 D_1 + m_1 D_0,
+//   f_2 f_3 = q - c t + g t^2 likewise;  U = q + g/3, V = q/3 + g/5:
+//   mean f_0 f_1 f_2 f_3 = p U + e V + b c / 3,
+//   mean f_1 f_2 f_3     = m_1 U + D_1 c / 3            (leave-one-out of 0),
+//   mean t f_1 f_2 f_3   = -(m_1 c / 3 + D_1 V),
+// and the in-bin weight (e_{k+1} - x) / h is linear in t, so its integral
+// against a leave-one-out product takes the last two.  Every lane runs the
+// same steps; row reads at crossings are predicated, partials are stored when
+// a neighbour leaves a bin (or the centre leaves one of its own).
+//
+// Bound by instruction issue and the FP32 pipe at two CTAs per SM (the rows'
+// shared memory).  One running partial per neighbour, A = C(start of its bin)
+// + in-bin integral, scaled by the centre's weight, is stored as it is and
+// restarted at C; the rows carry 1/h, whose 0 also says that the walker is
+// not inside a bin.  2048 x 2048 vertices, 16 bins: 2.83 -> 2.31 ms (three
+// Gauss-Legendre nodes, the partial in two parts and a width per walker
+// before).
 
 // the bin width of the rows of a support of width w (as hist_rows_build)
 __device__ __forceinline__ float rows_bin_width(float w, int B) {
   return (B & (B - 1)) == 0 ? w * (1.f / (float)B) : w / (float)B;
 }
 
-// a 4-byte global store that happens only where p holds (one predicated
-// instruction, no branch); the address is not touched where p is false
-__device__ __forceinline__ void stg_if(bool p, float *ptr, float v) {
+// One neighbour's crossing in the adjoint walk, without a branch: if its
+// next edge nx is at or below x1, store A (its partial of the bin it leaves)
+// at optr if it was inside a bin (r.y = 1/h, 0 outside), move optr to the
+// next bin's partial, restart A at C and read the next row into r.
+template <unsigned stride>
+__device__ __forceinline__ void adj_cross(float nx, float x1, float *&optr, long long qs, float C,
+                                          float &A, uint32_t &addr, float4 &r) {
   asm volatile(
-      "{\n .reg .pred q;\n setp.ne.b32 q, %2, 0;\n @q st.global.f32 [%0], %1;\n}" ::"l"(ptr),
-      "f"(v), "r"((int)p)
+      "{\n .reg .pred q, e;\n"
+      " setp.le.f32 q, %7, %8;\n"
+      " setp.ne.and.f32 e, %1, 0f00000000, q;\n"
+      " @e st.global.f32 [%4], %6;\n"
+      " @q add.s64 %4, %4, %9;\n"
+      " @q mov.f32 %6, %10;\n"
+      " @q ld.shared.v4.f32 {%0, %1, %2, %3}, [%5];\n"
+      " @q add.u32 %5, %5, %11;\n}"
+      : "+f"(r.x), "+f"(r.y), "+f"(r.z), "+f"(r.w), "+l"(optr), "+r"(addr), "+f"(A)
+      : "f"(nx), "f"(x1), "l"(qs * (long long)sizeof(float)), "f"(C), "n"(stride)
       : "memory");
 }
 
-// One neighbour's crossing in the adjoint walk, without a branch: if its
-// next edge nx is at or below x1 -- store `val` (its partial of the bin it
-// leaves) at optr if it was inside a bin (ihe != 0), move optr to the next
-// bin's partial, restart Cs = C and inb = 0, read the next row into r (and
-// advance addr), and set ihe to 1/h inside a bin (ih) or 0 beyond the
-// support (the beyond row's next edge is kFar).
+// The centre's crossing: if the next edge of its bin is at or below x1, store
+// its partial `own` of that bin at optr, move on and restart it.
 template <unsigned stride>
-__device__ __forceinline__ void adj_cross(float nx, float x1, float val, float *&optr,
-                                          long long qs, float C, float &Cs, float &inb,
-                                          uint32_t &addr, float4 &r, float ih, float &ihe) {
+__device__ __forceinline__ void adj_cross_centre(float x1, float *&optr, long long qs, float &own,
+                                                 uint32_t &addr, float2 &dc) {
   asm volatile(
-      "{\n .reg .pred q, e, n;\n"
-      " setp.le.f32 q, %9, %10;\n"
-      " setp.ne.and.f32 e, %8, 0f00000000, q;\n"
-      " @e st.global.f32 [%4], %11;\n"
-      " @q add.s64 %4, %4, %12;\n"
-      " @q mov.f32 %6, %13;\n"
-      " @q mov.f32 %7, 0f00000000;\n"
-      " @q ld.shared.v4.f32 {%0, %1, %2, %3}, [%5];\n"
-      " @q add.u32 %5, %5, %14;\n"
-      " setp.lt.and.f32 n, %3, 0f7E61B1E6, q;\n"
-      " @q selp.f32 %8, %15, 0f00000000, n;\n}"
-      : "+f"(r.x), "+f"(r.y), "+f"(r.z), "+f"(r.w), "+l"(optr), "+r"(addr), "+f"(Cs),
-        "+f"(inb), "+f"(ihe)
-      : "f"(nx), "f"(x1), "f"(val), "l"(qs * (long long)sizeof(float)), "f"(C), "n"(stride),
-        "f"(ih)
+      "{\n .reg .pred q;\n"
+      " setp.le.f32 q, %1, %5;\n"
+      " @q st.global.f32 [%2], %4;\n"
+      " @q add.s64 %2, %2, %6;\n"
+      " @q mov.f32 %4, 0f00000000;\n"
+      " @q ld.shared.v2.f32 {%0, %1}, [%3];\n"
+      " @q add.u32 %3, %3, %7;\n}"
+      : "+f"(dc.x), "+f"(dc.y), "+l"(optr), "+r"(addr), "+f"(own)
+      : "f"(x1), "l"(qs * (long long)sizeof(float)), "n"(stride)
       : "memory");
 }
 
@@ -898,128 +913,108 @@ __device__ __forceinline__ void hist_adj_walk(const float *sm, const float4 *R4,
     return;
   }
   HistRowWalker nw[4];
-  // per neighbour: C = int_0^x pdf_1 LOO, Cs = C at the start of its current
-  // bin, inb = the in-bin integral of that bin, ihe = 1/h inside a bin (0
-  // before or beyond its support, and for a point mass), kb = its bin (-1
-  // before the support, B beyond; a point mass moves from -1 to 0 at its
-  // position and stays there)
-  float2 C01 = {0.f, 0.f}, C23 = {0.f, 0.f}, inb01 = {0.f, 0.f}, inb23 = {0.f, 0.f};
-  float Cs[4] = {0.f, 0.f, 0.f, 0.f}, ih[4], ihe[4];
-  int kb[4];
-  bool pm[4];
+  // per neighbour: C = int_0^x pdf_1 LOO, A = C at the start of its current
+  // bin + the in-bin integral of that bin (both times wv); its bin (-1 before
+  // the support, B beyond; a point mass moves from -1 to 0 at its position
+  // and stays there) follows from the address of its next row
+  float2 C02 = {0.f, 0.f}, C13 = {0.f, 0.f};
+  float A[4] = {0.f, 0.f, 0.f, 0.f};
   float *optr[4];  // the partial of neighbour i's current bin (used inside a bin only)
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    pm[i] = false;
-    ih[i] = ihe[i] = 0.f;
     optr[i] = outc;
     if (!present[i]) {
       nw[i].init_absent();
-      kb[i] = B;
+      nw[i].r.y = 0.f;  // never inside a bin
       continue;
     }
     const float lo = sm[nl[i]], hi = sm[HALO + nl[i]];
-    pm[i] = lo == hi;
-    const float h = pm[i] ? 0.f : rows_bin_width(hi - lo, B);
-    ih[i] = pm[i] ? 0.f : frcp(h);
     nw[i].init(R4 + nl[i], lo - lo1, sm[2 * HALO + nl[i]]);
-    const int j = nw[i].seek0<RS>(R4 + nl[i], B, h);
-    kb[i] = j - 1;
-    ihe[i] = (kb[i] >= 0 && kb[i] < B) ? ih[i] : 0.f;
-    optr[i] = out(1 + i, 0) + (long long)kb[i] * qstride;
+    const int j = nw[i].seek0<RS, true>(R4 + nl[i], B, lo == hi ? 0.f : rows_bin_width(hi - lo, B));
+    optr[i] = out(1 + i, 0) + (long long)(j - 1) * qstride;
     // bins entirely below the centre's support: their survival is 0 there
-    if (!pm[i])
+    if (lo != hi)
       for (int q = 0; q < j - 1; ++q) *out(1 + i, q) = 0.f;
   }
-  const float ih1 = frcp(rows_bin_width(W1, B));
-  uint32_t addr_c = static_cast<uint32_t>(__cvta_generic_to_shared(R4 + l + RS)) + 8u;
+  const uint32_t row1_c = static_cast<uint32_t>(__cvta_generic_to_shared(R4 + l + RS)) + 8u;
+  uint32_t addr_c = row1_c;
   float2 dc;  // (density, next edge) of the centre's current bin
   {
     const float4 t = R4[l];
     dc = make_float2(t.z, t.w);
   }
-  int jc = 0;
+  float *optr_c = out(0, 0);
   float own = 0.f;
-  const float wvh = wv * ih1;
+  const float wvh = wv * frcp(rows_bin_width(W1, B));
   float x0 = 0.f;
   const int max_steps = 5 * (B + 1) + 4;
+  const float2 third = make_float2(1.f / 3.f, 1.f / 3.f), fifth = make_float2(0.2f, 0.2f);
 #pragma unroll 1
   for (int step = 0; step < max_steps && x0 < W1; ++step) {
     float e[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) e[i] = nw[i].nx();
-    const float x1 = fminf(fminf(fminf(e[0], e[1]), fminf(e[2], e[3])), dc.y);
-    const float d = x1 - x0, a = d * dc.x;
-    // the four factors in the pairs (0, 2) and (1, 3): values at x0 (g0),
-    // their change over the piece (dg); in-bin weights (e - x) / h at x0
-    // (w0) and their change (dw)
+    const float x1 = fmin5(e[0], e[1], e[2], e[3], dc.y);
+    const float d = x1 - x0, hd = 0.5f * d, xm = x0 + hd;
+    const float2 hh = make_float2(hd, hd), nh = make_float2(-hd, -hd), nx2 = make_float2(-xm, -xm);
+    // neighbours in the pairs (0, 2) and (1, 3): middle values m, half falls
+    // D, in-bin weights at the middle w and their half falls v
+    const float2 zA = make_float2(nw[0].r.z, nw[2].r.z), zB = make_float2(nw[1].r.z, nw[3].r.z);
     const float2 gA = make_float2(nw[0].r.x, nw[2].r.x), gB = make_float2(nw[1].r.x, nw[3].r.x);
-    const float2 sA = make_float2(-nw[0].r.z, -nw[2].r.z), sB = make_float2(-nw[1].r.z, -nw[3].r.z);
-    const float2 dd = make_float2(d, d);
-    const float2 dgA = __fmul2_rn(sA, dd), dgB = __fmul2_rn(sB, dd);
-    const float2 ihA = make_float2(ihe[0], ihe[2]), ihB = make_float2(ihe[1], ihe[3]);
-    const float2 w0A = __fmul2_rn(__fadd2_rn(make_float2(e[0], e[2]), make_float2(-x0, -x0)), ihA);
-    const float2 w0B = __fmul2_rn(__fadd2_rn(make_float2(e[1], e[3]), make_float2(-x0, -x0)), ihB);
-    const float2 dwA = __fmul2_rn(ihA, make_float2(-d, -d)), dwB = __fmul2_rn(ihB, make_float2(-d, -d));
-    // 3-point Gauss-Legendre on [0, 1]: nodes 1/2 -+ sqrt(3/5)/2, weights 5/18, 8/18
-    float so = 0.f;
-    float2 scA = {0.f, 0.f}, scB = {0.f, 0.f}, siA = {0.f, 0.f}, siB = {0.f, 0.f};
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      const float tq = q == 0 ? 0.11270166537925831f : (q == 1 ? 0.5f : 0.88729833462074169f);
-      const float wq = q == 1 ? 8.f / 18.f : 5.f / 18.f;
-      const float2 tt = make_float2(tq, tq), ww = make_float2(wq, wq);
-      const float2 fA = __ffma2_rn(dgA, tt, gA), fB = __ffma2_rn(dgB, tt, gB);  // (f0,f2),(f1,f3)
-      const float2 P = __fmul2_rn(fA, fB);                                       // (p01, p23)
-      const float2 Ps = make_float2(P.y, P.x);                                   // (p23, p01)
-      // leave-one-out products: (L0, L2) = (f1 p23, f3 p01), (L1, L3) = (f0 p23, f2 p01)
-      const float2 wLA = __fmul2_rn(ww, __fmul2_rn(fB, Ps));
-      const float2 wLB = __fmul2_rn(ww, __fmul2_rn(fA, Ps));
-      so = fmaf(wq, P.x * P.y, so);
-      scA = __fadd2_rn(scA, wLA);
-      scB = __fadd2_rn(scB, wLB);
-      siA = __ffma2_rn(__ffma2_rn(dwA, tt, w0A), wLA, siA);
-      siB = __ffma2_rn(__ffma2_rn(dwB, tt, w0B), wLB, siB);
-    }
-    own = fmaf(d, so, own);
+    const float2 iA = make_float2(nw[0].r.y, nw[2].r.y), iB = make_float2(nw[1].r.y, nw[3].r.y);
+    const float2 mA = __ffma2_rn(zA, nh, gA), mB = __ffma2_rn(zB, nh, gB);
+    const float2 DA = __fmul2_rn(zA, hh), DB = __fmul2_rn(zB, hh);
+    const float2 vA = __fmul2_rn(iA, hh), vB = __fmul2_rn(iB, hh);
+    const float2 wA = __fmul2_rn(__fadd2_rn(make_float2(e[0], e[2]), nx2), iA);
+    const float2 wB = __fmul2_rn(__fadd2_rn(make_float2(e[1], e[3]), nx2), iB);
+    // (01 | 23): products, cross terms / 3, U, V
+    const float2 p = __fmul2_rn(mA, mB), g = __fmul2_rn(DA, DB);
+    const float2 b = __ffma2_rn(mA, DB, __fmul2_rn(mB, DA)), b3 = __fmul2_rn(b, third);
+    const float2 U = __ffma2_rn(g, third, p), V = __ffma2_rn(p, third, __fmul2_rn(g, fifth));
+    own = fmaf(d * wvh, fmaf(p.x, U.y, fmaf(g.x, V.y, b.x * b3.y)), own);
+    // the other pair's, times the centre's density, weight and the width
+    const float a = (d * dc.x) * wv;
     const float2 aa = make_float2(a, a);
-    // back to the neighbour order (0, 1) and (2, 3)
-    C01 = __ffma2_rn(aa, make_float2(scA.x, scB.x), C01);
-    C23 = __ffma2_rn(aa, make_float2(scA.y, scB.y), C23);
-    inb01 = __ffma2_rn(aa, make_float2(siA.x, siB.x), inb01);
-    inb23 = __ffma2_rn(aa, make_float2(siA.y, siB.y), inb23);
-    float C[4] = {C01.x, C01.y, C23.x, C23.y}, inb[4] = {inb01.x, inb01.y, inb23.x, inb23.y};
-    // crossings: a neighbour leaving bin k stores its partial C(e_k) + in-bin
+    const float2 Uo = __fmul2_rn(aa, make_float2(U.y, U.x));
+    const float2 Vo = __fmul2_rn(aa, make_float2(V.y, V.x));
+    const float2 bo = __fmul2_rn(aa, make_float2(b3.y, b3.x));
+    // leave-one-out integrals of (0, 2) from the factors (1, 3), and back
+    const float2 sA = __ffma2_rn(mB, Uo, __fmul2_rn(DB, bo));
+    const float2 sB = __ffma2_rn(mA, Uo, __fmul2_rn(DA, bo));
+    const float2 tA = __ffma2_rn(mB, bo, __fmul2_rn(DB, Vo));
+    const float2 tB = __ffma2_rn(mA, bo, __fmul2_rn(DA, Vo));
+    C02 = __fadd2_rn(C02, sA);
+    C13 = __fadd2_rn(C13, sB);
+    const float2 a02 = __ffma2_rn(vA, tA, __ffma2_rn(wA, sA, make_float2(A[0], A[2])));
+    const float2 a13 = __ffma2_rn(vB, tB, __ffma2_rn(wB, sB, make_float2(A[1], A[3])));
+    A[0] = a02.x; A[2] = a02.y; A[1] = a13.x; A[3] = a13.y;
+    const float C[4] = {C02.x, C13.x, C02.y, C13.y};
+    // crossings: a neighbour leaving bin k stores its partial
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       nw[i].r.x = fmaf(-nw[i].r.z, d, nw[i].r.x);
-      adj_cross<(unsigned)(RS * 16)>(e[i], x1, wv * (Cs[i] + inb[i]), optr[i], qstride, C[i],
-                                     Cs[i], inb[i], nw[i].addr, nw[i].r, ih[i], ihe[i]);
+      adj_cross<(unsigned)(RS * 16)>(e[i], x1, optr[i], qstride, C[i], A[i], nw[i].addr, nw[i].r);
     }
-    inb01 = make_float2(inb[0], inb[1]);
-    inb23 = make_float2(inb[2], inb[3]);
-    {
-      const bool cr = dc.y <= x1;
-      stg_if(cr && jc < B, out(0, jc), wvh * own);
-      own = cr ? 0.f : own;
-      jc += cr ? 1 : 0;
-      lds64_cross<(unsigned)(RS * 16)>(dc.y, x1, addr_c, dc);
-    }
+    adj_cross_centre<(unsigned)(RS * 16)>(x1, optr_c, qstride, own, addr_c, dc);
     x0 = x1;
   }
-  if (jc < B) *out(0, jc) = wvh * own;
+  const int jc = (int)((addr_c - row1_c) / (uint32_t)(RS * 16));  // the bin the centre ended in
+  if (jc < B) *out(0, jc) = own;
   for (int q = jc + 1; q < B; ++q) *out(0, q) = 0.f;
-  const float C[4] = {C01.x, C01.y, C23.x, C23.y}, inb[4] = {inb01.x, inb01.y, inb23.x, inb23.y};
+  const float C[4] = {C02.x, C13.x, C02.y, C13.y};
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     if (!present[i]) continue;
-    kb[i] = (int)((optr[i] - out(1 + i, 0)) / qstride);  // the bin the walker ended in
-    if (kb[i] >= 0 && kb[i] < B) *out(1 + i, kb[i]) = wv * (Cs[i] + inb[i]);
+    // the bin the walker ended in
+    const uint32_t row0 = static_cast<uint32_t>(__cvta_generic_to_shared(R4 + nl[i]));
+    const int kb = (int)((nw[i].addr - row0) / (uint32_t)(RS * 16)) - 1;
+    const bool pm = sm[nl[i]] == sm[HALO + nl[i]];
+    if (kb >= 0 && kb < B) *out(1 + i, kb) = A[i];
     // bins entirely above the walk: their survival is 1 on the whole support
     // (a point mass: every mass partial is the integral below its position,
-    // Cs once it has been reached, else the whole integral)
-    const float above = pm[i] && kb[i] >= 0 ? Cs[i] : C[i];
-    for (int q = (kb[i] < 0 ? 0 : kb[i] + 1); q < B; ++q) *out(1 + i, q) = wv * above;
+    // A once it has been reached, else the whole integral)
+    const float above = pm && kb >= 0 ? A[i] : C[i];
+    for (int q = (kb < 0 ? 0 : kb + 1); q < B; ++q) *out(1 + i, q) = above;
   }
 }
 
@@ -1118,7 +1113,7 @@ __global__ void __launch_bounds__(NTHREADS, 2)
     __threadfence();
     slot_sm = got;
   }
-  hist_rows_from_params_tile<HALO, RS, RB, HX, true>(f, sm, R4, ty0, tx0, ylim, B, mirrored);
+  hist_rows_from_params_tile<HALO, RS, RB, HX, true, true>(f, sm, R4, ty0, tx0, ylim, B, mirrored);
   __syncthreads();
   const int slot = slot_sm;
   const int v = threadIdx.x;

@@ -1389,7 +1389,8 @@ struct HistRowWalker {
   // comes from -lam / h and is checked against the edges of the rows), and set G
   // and F to their values at 0.  Returns the number of edges crossed (a
   // point mass: 1), 0 if the first edge is above 0.
-  template <int RS>
+  // ADJ: rows of the adjoint, whose second entry is not a CDF (left as read).
+  template <int RS, bool ADJ = false>
   __device__ __forceinline__ int seek0(const float4 *row0, int B, float h) {
     if (nx() > 0.f) return 0;  // the first edge is above 0 (also: absent)
     int j = 1;               // edges e_0 .. e_{j-1} are at or below 0
@@ -1407,7 +1408,7 @@ struct HistRowWalker {
     // on the segment that starts at el <= 0: G(x) = S - slope (x - el) and
     // F(x) = T - S + slope (x - el), taken at x = 0
     r.x = fmaf(r.z, el, r.x);
-    r.y = fmaf(-r.z, el, r.y);
+    if constexpr (!ADJ) r.y = fmaf(-r.z, el, r.y);
     addr = static_cast<uint32_t>(__cvta_generic_to_shared(row0 + j * RS));
     return j;
   }

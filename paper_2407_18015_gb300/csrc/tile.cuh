@@ -470,8 +470,10 @@ struct HistParamRegs {
 
 // Per-bin rows, lo, hi, total and status of one staged vertex from its
 // parameters in registers; the same rows and status as hist_row_table
-// builds from a parameter tile.
-template <int HALO, int RS, int RB>
+// builds from a parameter tile.  ADJ (the adjoint, which walks the survivals
+// alone): the second entry of a row is 1 / h on a bin and 0 beyond the
+// support instead of T - S_k.
+template <int HALO, int RS, int RB, bool ADJ = false>
 __device__ __forceinline__ void hist_rows_build_regs(const HistParamRegs<RB> &P, float *sm,
                                                      float4 *R, int l, int B) {
   const float a = P.a, b = P.b;
@@ -487,7 +489,7 @@ __device__ __forceinline__ void hist_rows_build_regs(const HistParamRegs<RB> &P,
     }
   }
   R += l;
-  const float4 beyond = make_float4(0.f, t, 0.f, kFar);
+  const float4 beyond = make_float4(0.f, ADJ ? 0.f : t, 0.f, kFar);
   if (a == b) {
 #pragma unroll
     for (int k = 0; k <= RB; ++k)
@@ -502,7 +504,8 @@ __device__ __forceinline__ void hist_rows_build_regs(const HistParamRegs<RB> &P,
       if (k < B) {
         c += P.m[k];
         const float sn = k + 1 < B ? t - c : 0.f;
-        R[k * RS] = make_float4(sk, t - sk, (sk - sn) * ih, k + 1 < B ? (float)(k + 1) * h : w);
+        R[k * RS] = make_float4(sk, ADJ ? ih : t - sk, (sk - sn) * ih,
+                                k + 1 < B ? (float)(k + 1) * h : w);
         sk = sn;
       }
     }
@@ -522,7 +525,7 @@ __device__ __forceinline__ void hist_rows_build_regs(const HistParamRegs<RB> &P,
 // bins: forward from parameters 1.11 -> 1.06 ms, adjoint 2.85 -> 2.83 ms);
 // else one vertex after another (the 8-bin forward at four CTAs per SM:
 // 0.53 ms, against 0.57 batched).
-template <int HALO, int RS, int RB, int HX, bool BATCH>
+template <int HALO, int RS, int RB, int HX, bool BATCH, bool ADJ = false>
 __device__ __forceinline__ void hist_rows_from_params_tile(const Field &f, float *sm, float4 *R,
                                                            int ty0, int tx0, int ylim, int B,
                                                            bool mirrored) {
@@ -533,7 +536,7 @@ __device__ __forceinline__ void hist_rows_from_params_tile(const Field &f, float
       if (gy < 0 || gy >= ylim || gx < 0 || gx >= f.W) continue;
       HistParamRegs<RB> P;
       P.load(f, (long long)gy * f.W + gx, B, mirrored);
-      hist_rows_build_regs<HALO, RS, RB>(P, sm, R, l, B);
+      hist_rows_build_regs<HALO, RS, RB, ADJ>(P, sm, R, l, B);
     }
     return;
   }
@@ -550,7 +553,7 @@ __device__ __forceinline__ void hist_rows_from_params_tile(const Field &f, float
   }
 #pragma unroll
   for (int p = 0; p < PER; ++p)
-    if (in[p]) hist_rows_build_regs<HALO, RS, RB>(P[p], sm, R, threadIdx.x + p * NTHREADS, B);
+    if (in[p]) hist_rows_build_regs<HALO, RS, RB, ADJ>(P[p], sm, R, threadIdx.x + p * NTHREADS, B);
 }
 
 // ---------------------------------------------------------------------------
