@@ -18,7 +18,7 @@ __device__ __forceinline__ float qnan() { return __int_as_float(0x7fc00000); }
 // scratch of the walk ordering (buckets, then two 16-bit arrays of TYv x 32)
 __host__ __device__ constexpr long long tile_floats(int model, int B, int TYv) {
   const long long halo = (long long)(TYv + 2) * 34;
-  return model == kSemi   ? (2 + 2LL * B) * halo
+  return model == kSemi   ? semi_rows(B) * halo
          : model == kHist ? hist_rows(B) * halo + kSortBuckets + TYv * 32
                           : 2 * halo;
 }
@@ -1023,7 +1023,7 @@ __device__ __forceinline__ uint8_t check_params(const float *sm, int l, int B, f
   uint8_t st = a > b ? V_BAD : (a == b ? V_DEGENERATE : 0);
   float t = 0.f;
   for (int q = 0; q < B; ++q) {
-    const float w = sm[(2 + q) * HALO + l];
+    const float w = sm[(3 + 2 * q) * HALO + l];  // the estimator's rows
     if (!isfinite(w)) st |= V_NONFINITE;
     else if (w < 0.f) st |= V_BAD;
     t += w;
@@ -1145,13 +1145,24 @@ __device__ __forceinline__ void integrate_tile(const Field &f, int ty0, int tx0,
     __syncthreads();
   }
   if constexpr (MODEL == kSemi) {
-    // running mass sums C_1..C_B of every staged vertex, in bin order
+    // the rows of semi_rows from the masses staged in rows 2 .. 1 + B: masses
+    // moved up to every other row (from the last: a mass moves to a row
+    // above those not yet moved), then the running sums in bin order
     for (int l = threadIdx.x; l < HALO; l += NTHREADS) {
+      for (int q = f.B - 1; q >= 0; --q) sm[(3 + 2 * q) * HALO + l] = sm[(2 + q) * HALO + l];
       float c = 0.f;
       for (int q = 0; q < f.B; ++q) {
-        c += sm[(2 + q) * HALO + l];
-        sm[(2 + f.B + q) * HALO + l] = c;
+        sm[(2 + 2 * q) * HALO + l] = c;
+        c += sm[(3 + 2 * q) * HALO + l];
       }
+      sm[(2 + 2 * f.B) * HALO + l] = c;
+      sm[(3 + 2 * f.B) * HALO + l] = 0.f;
+    }
+    // what an absent neighbour reads, in the corner's rows (this thread built
+    // them)
+    if (threadIdx.x == 0) {
+      sm[2 * HALO] = 1.f;
+      sm[3 * HALO] = 0.f;
     }
     __syncthreads();
   }
@@ -1205,12 +1216,14 @@ __device__ __forceinline__ void integrate_tile(const Field &f, int ty0, int tx0,
       const float lo1 = sm[l];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        nb[i].off = nl[i];
+        nb[i].off = 2 * HALO + nl[i];
         nb[i].T = T[i];
-        if (!present[i]) {
+        if (!present[i]) {  // F = 1, G = T - F = 1 (semi_cdf)
           nb[i].kind = 0;
           nb[i].lam = 0.f;
           nb[i].ih = 0.f;
+          nb[i].T = 2.f;
+          nb[i].off = 2 * HALO;
           continue;
         }
         const float lo = sm[nl[i]], hi = sm[HALO + nl[i]];
@@ -1220,9 +1233,9 @@ __device__ __forceinline__ void integrate_tile(const Field &f, int ty0, int tx0,
       }
       const PhiloxKeys K(f.seed_lo, f.seed_hi);
       if (!SADDLE || has_saddle)
-        semi_vertex<HALO, SADDLE>(sm + 2 * HALO, sm + (2 + f.B) * HALO, l, lo1, sm[HALO + l], nb,
-                                  f.B, f.samples, K, (uint32_t)((long long)gy * f.W + gx),
-                                  f.field_id, sg, pmin, pmax, psad);
+        semi_vertex<HALO, SADDLE>(sm, l, lo1, sm[HALO + l], nb, f.B, f.samples, K,
+                                  (uint32_t)((long long)gy * f.W + gx), f.field_id, sg, pmin,
+                                  pmax, psad);
       if (!SADDLE && f.boundary == 1 && k < 4) pmin = pmax = 0.f;
     } else if (MODEL == kUniform) {
       UniParams cp{sm[l], sm[HALO + l]}, nb[4];
