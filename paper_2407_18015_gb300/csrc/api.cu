@@ -275,7 +275,7 @@ static int probability_impl(ucp_ctx *ctx, const float *ens, const float *params,
 }
 
 // minimum / maximum with a larger stencil: statistics pass into workspace
-// (from members), tail tables (histogram), then one thread per vertex
+// (from members), tail tables (histograms of many bins), then the vertices
 static int stencil_impl(ucp_ctx *ctx, const float *ens, const float *params, int N, int H,
                         int W, const ucp_model_desc *desc, unsigned cptypes, float *out_min,
                         float *out_max, uint8_t *vertex_status, cudaStream_t stream) {
@@ -284,7 +284,8 @@ static int stencil_impl(ucp_ctx *ctx, const float *ens, const float *params, int
   const int B = desc->bins;
   const int P = param_planes(desc->model, B);
   const size_t fit_floats = ens ? (size_t)P * V : 0;
-  const size_t tab_floats = desc->model == UCP_HISTOGRAM ? (size_t)(B + 4) * V : 0;
+  const bool table = desc->model == UCP_HISTOGRAM && !stencil_hist_tiles(desc->stencil, B);
+  const size_t tab_floats = table ? (size_t)(B + 4) * V : 0;
   int rc = ucp_ensure_work(ctx, (fit_floats + tab_floats) * sizeof(float) + 256);
   if (rc) return rc;
   float *work = static_cast<float *>(ctx->work);
@@ -301,7 +302,7 @@ static int stencil_impl(ucp_ctx *ctx, const float *ens, const float *params, int
     params = work;
   }
   float *tab = nullptr;
-  if (e == cudaSuccess && desc->model == UCP_HISTOGRAM) {
+  if (e == cudaSuccess && table) {
     tab = work + fit_floats;
     e = launch_hist_table(params, V, B, tab, ctx->sm_count, stream);
   }

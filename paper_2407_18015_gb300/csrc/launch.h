@@ -70,7 +70,8 @@ cudaError_t launch_mvn_mc(const Field &f, bool from_members, int samples, uint64
                           uint32_t field_id, cudaStream_t s);
 
 // Larger neighbour sets (stencil.cu): one thread per vertex of a D x H x W
-// grid, parameters [P][D][H][W] in global memory, histogram tail tables
+// grid, parameters [P][D][H][W] in global memory; histograms of too many bins
+// for shared-memory rows (stencil_hist_tiles false) also tail tables
 // [D*H*W][B+4] (see stencil.cuh).
 struct StencilField {
   const float *params;  // [P][D][H][W]
@@ -83,6 +84,7 @@ struct StencilField {
   int boundary;
   unsigned cptypes;
 };
+bool stencil_hist_tiles(int stencil, int B);
 cudaError_t launch_hist_table(const float *params, long long V, int B, float *tab, int sm_count,
                               cudaStream_t s);
 cudaError_t launch_stencil(const StencilField &f, int model, int stencil, int sm_count,

@@ -342,7 +342,8 @@ __device__ __forceinline__ void epan_vertex_k(EpanParams c, const EpanParams *nb
 }
 
 // ---------------------------------------------------------------------------
-// histogram: tail tables in global memory, one row of R = B + 4 floats per
+// histogram of many bins (see stencil_hist_tiles): tail tables in global
+// memory, one row of R = B + 4 floats per
 // vertex: S_0..S_{B+1} (S_k = T - (m_0 + ... + m_{k-1}), S_B = S_{B+1} = 0,
 // all 0 for a point mass), the total mass T, the status bits
 
@@ -440,6 +441,119 @@ __device__ __forceinline__ void hist_walk_k(const float *tab, long long crow, in
   }
   pmin = fmaxf(acc.x, 0.f);
   pmax = fmaxf(acc.y, 0.f);
+}
+
+// Mean over [-1, 1] of the product of K = 6 or 8 linear factors m_i - D_i t,
+// from their middle values and half falls: pairs of factors are quadratics p -
+// b t + e t^2, two pairs a quartic, and the mean of a product of polynomials
+// is the sum of its even coefficients over 1, 3, 5, ... .  Every term is a
+// product of non-negative numbers.  O: the arithmetic of one or both types
+// (HistWalkOps); with both, the odd coefficients of F carry the opposite
+// sign, which drops out (they meet in pairs).
+template <int K, typename O, typename V>
+__device__ __forceinline__ V linear_mean_k(const V *m, const V *D) {
+  static_assert(K == 6 || K == 8, "three or four pairs");
+  constexpr int P = K / 2;
+  V p[P], b[P], e[P];
+#pragma unroll
+  for (int j = 0; j < P; ++j) {
+    p[j] = O::mul(m[2 * j], m[2 * j + 1]);
+    e[j] = O::mul(D[2 * j], D[2 * j + 1]);
+    b[j] = O::fma(m[2 * j], D[2 * j + 1], O::mul(m[2 * j + 1], D[2 * j]));
+  }
+  const V c3 = O::all(1.f / 3.f), c5 = O::all(0.2f), c7 = O::all(1.f / 7.f);
+  // the quartic of two pairs: coefficients of 1, -t, t^2, -t^3, t^4
+  auto quartic = [&](int i, int j, V *q) {
+    q[0] = O::mul(p[i], p[j]);
+    q[1] = O::fma(p[i], b[j], O::mul(b[i], p[j]));
+    q[2] = O::fma(p[i], e[j], O::fma(b[i], b[j], O::mul(e[i], p[j])));
+    q[3] = O::fma(b[i], e[j], O::mul(e[i], b[j]));
+    q[4] = O::mul(e[i], e[j]);
+  };
+  V q[5];
+  quartic(0, 1, q);
+  if constexpr (K == 6) {
+    const V u0 = O::fma(e[2], c3, p[2]);
+    const V u2 = O::fma(p[2], c3, O::mul(e[2], c5));
+    const V u4 = O::fma(p[2], c5, O::mul(e[2], c7));
+    const V v = O::fma(q[3], c5, O::mul(q[1], c3));
+    return O::fma(q[0], u0, O::fma(q[2], u2, O::fma(q[4], u4, O::mul(v, b[2]))));
+  } else {
+    V r[5];
+    quartic(2, 3, r);
+    const V c9 = O::all(1.f / 9.f);
+    const V u0 = O::fma(r[2], c3, O::fma(r[4], c5, r[0]));
+    const V u2 = O::fma(r[0], c3, O::fma(r[2], c5, O::mul(r[4], c7)));
+    const V u4 = O::fma(r[0], c5, O::fma(r[2], c7, O::mul(r[4], c9)));
+    const V v1 = O::fma(r[1], c3, O::mul(r[3], c5));
+    const V v3 = O::fma(r[1], c5, O::mul(r[3], c7));
+    return O::fma(q[0], u0,
+                  O::fma(q[2], u2, O::fma(q[4], u4, O::fma(q[1], v1, O::mul(q[3], v3)))));
+  }
+}
+
+// hist_walk_pieces with K neighbours: the same rows, walkers and steps (every
+// lane runs the same instructions, the crossings predicated); MODE kWalkBoth,
+// kWalkMin or kWalkMax.
+template <int K, int RS, int MODE>
+__device__ __forceinline__ void hist_walk_rows_k(const float4 *crow, int B, float W1,
+                                                 HistRowWalker *nw, float &pmin, float &pmax) {
+  using O = HistWalkOps<MODE>;
+  using V = typename O::V;
+  if (!(W1 <= 1e38f)) {
+    pmin = pmax = __int_as_float(0x7fc00000);
+    return;
+  }
+  uint32_t addr_c = static_cast<uint32_t>(__cvta_generic_to_shared(crow + RS)) + 8u;
+  float2 dc;  // (density, next edge) of the centre's current bin
+  {
+    const float4 t = crow[0];
+    dc = make_float2(t.z, t.w);
+  }
+  V acc = O::all(0.f);
+  float x0 = 0.f;
+  const int max_steps = (K + 1) * (B + 1) + 4;
+#pragma unroll 1
+  for (int step = 0; step < max_steps && x0 < W1; ++step) {
+    float e[K];
+    float x1 = dc.y;
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+      e[i] = nw[i].nx();
+      x1 = fminf(x1, e[i]);
+    }
+    const float d = x1 - x0, hd = 0.5f * d;
+    V m[K], D[K];
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+      float4 &r = nw[i].r;
+      if constexpr (O::two) {
+        const float2 zz = make_float2(r.z, r.z), l = make_float2(r.x, r.y);
+        D[i] = __fmul2_rn(zz, make_float2(hd, hd));
+        m[i] = __ffma2_rn(zz, make_float2(-hd, hd), l);
+        const float2 v = __ffma2_rn(zz, make_float2(-d, d), l);
+        r.x = v.x;
+        r.y = v.y;
+      } else {
+        float &l = MODE == kWalkMin ? r.x : r.y;
+        D[i] = __fmul_rn(r.z, hd);
+        m[i] = __fmaf_rn(r.z, MODE == kWalkMin ? -hd : hd, l);
+        l = __fmaf_rn(r.z, MODE == kWalkMin ? -d : d, l);
+      }
+    }
+    acc = O::fma(O::all(__fmul_rn(d, dc.x)), linear_mean_k<K, O>(m, D), acc);
+#pragma unroll
+    for (int i = 0; i < K; ++i)
+      lds128_cross<(unsigned)(RS * 16)>(e[i], x1, nw[i].addr, nw[i].r);
+    lds64_cross<(unsigned)(RS * 16)>(dc.y, x1, addr_c, dc);
+    x0 = x1;
+  }
+  if constexpr (O::two) {
+    pmin = fmaxf(acc.x, 0.f);
+    pmax = fmaxf(acc.y, 0.f);
+  } else {
+    (MODE == kWalkMin ? pmin : pmax) = fmaxf(acc, 0.f);
+  }
 }
 
 // survival and CDF of a histogram neighbour (tail-table row) at a point v
