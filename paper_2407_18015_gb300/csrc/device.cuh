@@ -10,7 +10,8 @@
 //     piece, so the integral of the product is the Bernstein mean of its end
 //     values (no quadrature, all terms non-negative, no cancellation);
 //   - Epanechnikov: pdf_1 quadratic, G_n cubic, degree <= 14 on a piece,
-//     integrated exactly by 8-point Gauss-Legendre (exact to degree 15).
+//     integrated exactly by the Gauss-Legendre rule of the piece's degree (at
+//     most 8 points).
 // All arithmetic is FP32 in a vertex-local frame (the centre's lower support
 // end or mean is the origin), pieces are summed with Kahan compensation.
 #pragma once
@@ -74,6 +75,9 @@ __device__ __forceinline__ float fmax3_nan(float a, float b, float c) {
   asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
   return r;
 }
+
+// max(x, 0), NaN kept
+__device__ __forceinline__ float not_negative(float x) { return x < 0.f ? 0.f : x; }
 
 // Compensated (Kahan) summation: the running rounding error c is fed back
 // into the next addend.
@@ -494,11 +498,9 @@ __device__ __constant__ const float kGLx[4] = {0.18343464249564978f, 0.525532409
 __device__ __constant__ const float kGLw[4] = {0.36268378337836166f, 0.3137066458778869f,
                                                0.22238103445337443f, 0.10122853629037706f};
 
-// Gauss-Legendre rules on [-1, 1] with 2, 3, 5 and 6 nodes (all nodes,
+// Gauss-Legendre rules on [-1, 1] with 3, 5 and 6 nodes (all nodes,
 // ascending: the roots of P_n, weights 2 / ((1 - x^2) P_n'(x)^2)); the n-point
 // rule is exact for polynomials of degree <= 2n - 1.
-__device__ __constant__ const float kGL2x[2] = {-0.57735026918962573f, 0.57735026918962573f};
-__device__ __constant__ const float kGL2w[2] = {1.f, 1.f};
 __device__ __constant__ const float kGL3x[3] = {-0.7745966692414834f, 0.f, 0.7745966692414834f};
 __device__ __constant__ const float kGL3w[3] = {0.55555555555555569f, 0.88888888888888884f,
                                                 0.55555555555555569f};
@@ -514,10 +516,20 @@ __device__ __constant__ const float kGL6w[6] = {0.17132449237917027f, 0.36076157
                                                 0.46791393457269104f, 0.46791393457269104f,
                                                 0.36076157304813872f, 0.17132449237917027f};
 
-// node / weight q (ascending) of the NG-point rule, NG in {2, 3, 5, 6, 8}
+// nodes (positive half, ascending) and weights of the 16-point rule on
+// [-1, 1]: the roots of the Legendre polynomial P_16 and 2 / ((1 - x^2)
+// P_16'(x)^2)
+__device__ __constant__ const float kGL16x[8] = {
+    0.095012509837637441f, 0.28160355077925892f, 0.45801677765722737f, 0.61787624440264377f,
+    0.755404408355003f,    0.86563120238783176f, 0.9445750230732326f,  0.98940093499164994f};
+__device__ __constant__ const float kGL16w[8] = {
+    0.18945061045506864f, 0.18260341504492364f, 0.16915651939500265f, 0.14959598881657671f,
+    0.12462897125553407f, 0.095158511682492605f, 0.062253523938647456f, 0.027152459411754176f};
+
+// node / weight q (ascending) of the NG-point rule, NG in {3, 5, 6, 8, 16}
 template <int NG>
 __device__ __forceinline__ float gl_x(int q) {
-  if constexpr (NG == 2) return kGL2x[q];
+  if constexpr (NG == 16) return q < 8 ? -kGL16x[7 - q] : kGL16x[q - 8];
   else if constexpr (NG == 3) return kGL3x[q];
   else if constexpr (NG == 5) return kGL5x[q];
   else if constexpr (NG == 6) return kGL6x[q];
@@ -525,7 +537,7 @@ __device__ __forceinline__ float gl_x(int q) {
 }
 template <int NG>
 __device__ __forceinline__ float gl_w(int q) {
-  if constexpr (NG == 2) return kGL2w[q];
+  if constexpr (NG == 16) return q < 8 ? kGL16w[7 - q] : kGL16w[q - 8];
   else if constexpr (NG == 3) return kGL3w[q];
   else if constexpr (NG == 5) return kGL5w[q];
   else if constexpr (NG == 6) return kGL6w[q];
@@ -539,57 +551,86 @@ __device__ __forceinline__ float epan_surv(float u) {
   return 0.25f * q * q * (2.f + u);
 }
 
-// Piece J of epan_side: on [x[J], x[J+1]] the centre density (degree 2)
-// times the J started survivals (degree 3 each) has degree 2 + 3J, so the
-// n-point rule with 2n - 1 >= 2 + 3J is exact: n = 2, 3, 5, 6, 8.
+// Gauss-Legendre rule of a piece on which J survivals (degree 3 each) and the
+// centre density (degree 2) are polynomials: the n-point rule with 2n - 1 >=
+// 2 + 3J is exact (n = 3, 5, 6, 8 for J = 1..4; 16 for the J = 5..8 of larger
+// stencils).
 template <int J>
 struct EpanNodes {
-  static constexpr int value = J == 0 ? 2 : (J == 1 ? 3 : (J == 2 ? 5 : (J == 3 ? 6 : 8)));
+  static constexpr int value = J == 1 ? 3 : (J == 2 ? 5 : (J == 3 ? 6 : (J == 4 ? 8 : 16)));
 };
+__host__ __device__ constexpr float epan_scale4(int J) { return J == 0 ? 1.f : 0.25f * epan_scale4(J - 1); }
+
+// int over a piece (middle mid, half width half) of (1 - u^2) prod_{i<J} S_i,
+// u = x iw1 and S_i = q_i^2 (3 - q_i) / 4 the survival of factor i at q_i = 1 -
+// (its argument) in [0, 2].  On the piece q_i = qm_i - qd_i xi is linear in
+// the node xi, so a node takes one multiply-add per factor for q_i, and the
+// squares and the quarters are taken once per node and piece: 4 J + 4
+// operations per node, where each factor's argument, clamp and cubic on its
+// own took 7 J + 6 (Epanechnikov saddle of 500 x 500 x 20: 41 -> 24.6 us; three
+// models of 1024 x 1024 x 20: 222 -> 211 us).  Nodes in pairs, one per half of a float2 (packed FP32
+// instructions).
 template <int J>
-__device__ __forceinline__ void epan_pieces(const float *x, const float (*pay)[4], float iw1,
-                                            float c1, Kahan &acc) {
-  constexpr int NG = EpanNodes<J>::value;
-  const float x0 = x[J], x1 = x[J + 1];
-  const float half = 0.5f * (x1 - x0), mid = 0.5f * (x0 + x1);
-  // nodes in pairs, one per half of a float2 (packed FP32 instructions)
-  const float2 one2 = make_float2(1.f, 1.f);
-  float2 s2 = make_float2(0.f, 0.f);
+__device__ __forceinline__ float epan_piece(float mid, float half, float iw1, const float *qm,
+                                            const float *qd) {
+  const float um = mid * iw1, ud = half * iw1;
+  if constexpr (J == 0) {
+    // the mean of 1 - u^2
+    return 2.f * half * fmaf(-um, um, fmaf(-ud * (1.f / 3.f), ud, 1.f));
+  } else {
+    constexpr int NG = EpanNodes<J>::value;
+    const float2 one2 = make_float2(1.f, 1.f), three2 = make_float2(3.f, 3.f);
+    float2 s2 = make_float2(0.f, 0.f);
 #pragma unroll
-  for (int q = 0; q + 1 < NG; q += 2) {
-    const float2 xx = __ffma2_rn(make_float2(half, half),
-                                 make_float2(gl_x<NG>(q), gl_x<NG>(q + 1)), make_float2(mid, mid));
-    const float2 u1 = __fmul2_rn(xx, make_float2(iw1, iw1));
-    const float2 g = __ffma2_rn(make_float2(-u1.x, -u1.y), u1, one2);
-    float2 f = __fmul2_rn(make_float2(c1, c1), make_float2(fmaxf(g.x, 0.f), fmaxf(g.y, 0.f)));
+    for (int n = 0; n + 1 < NG; n += 2) {
+      const float2 xi = make_float2(gl_x<NG>(n), gl_x<NG>(n + 1));
+      const float2 u = __ffma2_rn(make_float2(ud, ud), xi, make_float2(um, um));
+      const float2 g = __ffma2_rn(make_float2(-u.x, -u.y), u, one2);
+      float2 Q = one2, T = one2;
 #pragma unroll
-    for (int i = 0; i < J; ++i) {
-      // epan_surv of both nodes, unclamped: on the piece where J factors
-      // have started, each started factor's u lies in [-1, 1] (the piece
-      // begins after the factor's start, and R is at most every present
-      // neighbour's end); absent and point-mass factors start at R and so
-      // only enter pieces of zero width
-      const float2 u = __fmul2_rn(__fadd2_rn(xx, make_float2(-pay[0][i], -pay[0][i])),
-                                  make_float2(pay[1][i], pay[1][i]));
-      const float2 qq = __fadd2_rn(one2, make_float2(-u.x, -u.y));
-      const float2 sv = __fmul2_rn(__fmul2_rn(make_float2(0.25f, 0.25f), __fmul2_rn(qq, qq)),
-                                   __fadd2_rn(make_float2(2.f, 2.f), u));
-      f = __fmul2_rn(f, sv);
+      for (int i = 0; i < J; ++i) {
+        const float2 q = __ffma2_rn(make_float2(-qd[i], -qd[i]), xi, make_float2(qm[i], qm[i]));
+        const float2 t = __fadd2_rn(three2, make_float2(-q.x, -q.y));
+        Q = i == 0 ? q : __fmul2_rn(Q, q);
+        T = i == 0 ? t : __fmul2_rn(T, t);
+      }
+      const float2 f = __fmul2_rn(__fmul2_rn(Q, Q), __fmul2_rn(T, g));
+      s2 = __ffma2_rn(make_float2(gl_w<NG>(n), gl_w<NG>(n + 1)), f, s2);
     }
-    s2 = __ffma2_rn(make_float2(gl_w<NG>(q), gl_w<NG>(q + 1)), f, s2);
-  }
-  float s = s2.x + s2.y;
-  if constexpr (NG & 1) {
-    constexpr int q = NG - 1;
-    const float xx = fmaf(half, gl_x<NG>(q), mid);
-    const float u1 = xx * iw1;
-    float f = c1 * fmaxf(fmaf(-u1, u1, 1.f), 0.f);
+    float s = s2.x + s2.y;
+    if constexpr (NG & 1) {
+      constexpr int n = NG - 1;
+      const float u = fmaf(ud, gl_x<NG>(n), um);
+      float Q = 1.f, T = fmaf(-u, u, 1.f);
 #pragma unroll
-    for (int i = 0; i < J; ++i) f *= epan_surv((xx - pay[0][i]) * pay[1][i]);
-    s = fmaf(gl_w<NG>(q), f, s);
+      for (int i = 0; i < J; ++i) {
+        const float q = fmaf(-qd[i], gl_x<NG>(n), qm[i]);
+        Q *= q;
+        T *= 3.f - q;
+      }
+      s = fmaf(gl_w<NG>(n) * (Q * Q), T, s);
+    }
+    return s * (half * epan_scale4(J));
   }
-  acc.add(s * half);
-  if constexpr (J < 4) epan_pieces<J + 1>(x, pay, iw1, c1, acc);
+}
+
+// Pieces J.. of epan_side: on [x[J], x[J+1]] the sorted factors 0..J-1 have
+// started.  A started factor's argument lies in [-1, 1] there (the piece
+// begins after the factor's start, and R is at most every present
+// neighbour's end); a factor that starts at R enters pieces of zero width
+// alone, where q is held at 2 (its survival at 1) so that nothing overflows.
+template <int J, int K, int NP>
+__device__ __forceinline__ void epan_pieces(const float *x, const float (*pay)[NP], float iw1,
+                                            Kahan &acc) {
+  const float half = 0.5f * (x[J + 1] - x[J]), mid = 0.5f * (x[J] + x[J + 1]);
+  float qm[J > 0 ? J : 1], qd[J > 0 ? J : 1];
+#pragma unroll
+  for (int i = 0; i < J; ++i) {
+    qm[i] = fminf(fmaf(-(mid - pay[0][i]), pay[1][i], 1.f), 2.f);
+    qd[i] = half * pay[1][i];
+  }
+  acc.add(epan_piece<J>(mid, half, iw1, qm, qd));
+  if constexpr (J < K) epan_pieces<J + 1, K, NP>(x, pay, iw1, acc);
 }
 
 // One-sided problem in the centre's frame (origin m1): centre pdf
@@ -610,10 +651,9 @@ __device__ __forceinline__ float epan_side(float w1, float L, float R, float al[
   sort4<2>(t, pay);
   const float x[6] = {L, t[0], t[1], t[2], t[3], R};
   const float iw1 = frcp(w1);
-  const float c1 = 0.75f * iw1;
   Kahan acc;
-  epan_pieces<0>(x, pay, iw1, c1, acc);
-  return acc.get();
+  epan_pieces<0, 4, 4>(x, pay, iw1, acc);
+  return not_negative(0.75f * iw1 * acc.get());
 }
 
 struct EpanParams {
@@ -685,16 +725,6 @@ __device__ __forceinline__ void epan_vertex(EpanParams c, const EpanParams *nb,
     pmax = epan_side(w1, -w1, R, al, d, iw);
   }
 }
-
-// nodes (positive half, ascending) and weights of the 16-point rule on
-// [-1, 1]: the roots of the Legendre polynomial P_16 and 2 / ((1 - x^2)
-// P_16'(x)^2)
-__device__ __constant__ const float kGL16x[8] = {
-    0.095012509837637441f, 0.28160355077925892f, 0.45801677765722737f, 0.61787624440264377f,
-    0.755404408355003f,    0.86563120238783176f, 0.9445750230732326f,  0.98940093499164994f};
-__device__ __constant__ const float kGL16w[8] = {
-    0.18945061045506864f, 0.18260341504492364f, 0.16915651939500265f, 0.14959598881657671f,
-    0.12462897125553407f, 0.095158511682492605f, 0.062253523938647456f, 0.027152459411754176f};
 
 // ---------------------------------------------------------------------------
 // independent Gaussians (the parametric model the paper compares with by
@@ -917,7 +947,9 @@ __device__ __forceinline__ float uniform_mixed(UniParams c, const UniParams *nb,
 }
 
 // Epanechnikov: the same, 8-point Gauss-Legendre on each piece (origin m1);
-// F_i(x) = epan_surv((m_i - x)/w_i) by the kernel's symmetry
+// F_i(x) = epan_surv((m_i - x)/w_i) by the kernel's symmetry, so both kinds
+// are q^2 (3 - q) / 4 with q falling (survival) or rising (CDF) in x.  A
+// factor is a polynomial or the constant 1 (q = 2) on all of a piece.
 __device__ __forceinline__ float epan_mixed(EpanParams c, const EpanParams *nb, const int *sg) {
   if (c.w == 0.f) {
     const float v = c.m;
@@ -934,18 +966,18 @@ __device__ __forceinline__ float epan_mixed(EpanParams c, const EpanParams *nb, 
   }
   const float w1 = c.w;
   float L = -w1, R = w1;
-  float bp[4], d[4], iw[4], sgn[4];
+  float bp[4], d[4], iw[4];  // iw: 1/w with the sign of q's fall; 0: the constant 1
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    bp[i] = kFar; d[i] = 0.f; iw[i] = 0.f; sgn[i] = 0.f;
+    bp[i] = kFar; d[i] = 0.f; iw[i] = 0.f;
     if (sg[i] == 0) continue;
     const float dn = nb[i].m - c.m, wn = nb[i].w;
     if (sg[i] > 0) {
       R = fminf(R, dn + wn);
-      if (wn > 0.f) { bp[i] = dn - wn; d[i] = dn; iw[i] = frcp(wn); sgn[i] = 1.f; }
+      if (wn > 0.f) { bp[i] = dn - wn; d[i] = dn; iw[i] = frcp(wn); }
     } else {
       L = fmaxf(L, dn - wn);
-      if (wn > 0.f) { bp[i] = dn + wn; d[i] = dn; iw[i] = frcp(wn); sgn[i] = -1.f; }
+      if (wn > 0.f) { bp[i] = dn + wn; d[i] = dn; iw[i] = -frcp(wn); }
     }
   }
   if (!(R > L)) return 0.f;
@@ -955,41 +987,22 @@ __device__ __forceinline__ float epan_mixed(EpanParams c, const EpanParams *nb, 
   float none[1][4];
   sort4<0>(t, none);
   const float x[6] = {L, t[0], t[1], t[2], t[3], R};
-  const float iw1 = frcp(w1), c1 = 0.75f * iw1;
+  const float iw1 = frcp(w1);
   Kahan acc;
-  // the 8 nodes in the symmetric pairs (-x_k, x_k), which share the weight
-  // w_k: one pair per float2 (packed FP32 instructions, the same operations
-  // per node as the scalar form)
-  const float2 one2 = make_float2(1.f, 1.f), two2 = make_float2(2.f, 2.f);
 #pragma unroll
   for (int j = 0; j <= 4; ++j) {
     const float half = 0.5f * (x[j + 1] - x[j]), mid = 0.5f * (x[j] + x[j + 1]);
-    float2 s2 = make_float2(0.f, 0.f);
+    float qm[4], qd[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const float2 xx = __ffma2_rn(make_float2(half, half), make_float2(-kGLx[k], kGLx[k]),
-                                   make_float2(mid, mid));
-      const float2 u1 = __fmul2_rn(xx, make_float2(iw1, iw1));
-      const float2 g = __ffma2_rn(make_float2(-u1.x, -u1.y), u1, one2);
-      float2 f = __fmul2_rn(make_float2(c1, c1), make_float2(fmaxf(g.x, 0.f), fmaxf(g.y, 0.f)));
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if (sgn[i] == 0.f) continue;
-        // epan_surv of sgn (x - d) / w at both nodes
-        float2 u = __fmul2_rn(__fmul2_rn(make_float2(sgn[i], sgn[i]),
-                                         __fadd2_rn(xx, make_float2(-d[i], -d[i]))),
-                              make_float2(iw[i], iw[i]));
-        u = make_float2(fminf(fmaxf(u.x, -1.f), 1.f), fminf(fmaxf(u.y, -1.f), 1.f));
-        const float2 qq = __fadd2_rn(one2, make_float2(-u.x, -u.y));
-        const float2 sv = __fmul2_rn(__fmul2_rn(__fmul2_rn(make_float2(0.25f, 0.25f), qq), qq),
-                                     __fadd2_rn(two2, u));
-        f = __fmul2_rn(f, sv);
-      }
-      s2 = __ffma2_rn(make_float2(kGLw[k], kGLw[k]), f, s2);
+    for (int i = 0; i < 4; ++i) {
+      const float q = fmaf(-(mid - d[i]), iw[i], 1.f);
+      const bool one = iw[i] == 0.f || q >= 2.f;
+      qm[i] = one ? 2.f : q;
+      qd[i] = one ? 0.f : half * iw[i];
     }
-    acc.add((s2.x + s2.y) * half);
+    acc.add(epan_piece<4>(mid, half, iw1, qm, qd));
   }
-  return acc.get();
+  return not_negative(0.75f * iw1 * acc.get());
 }
 
 // saddle signs of the four slots (e, n, w, s) for t1, or all zero when the
