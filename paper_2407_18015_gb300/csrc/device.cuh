@@ -1066,12 +1066,6 @@ __device__ __forceinline__ uint4 philox_block(uint4 c, const PhiloxKeys &K) {
 __device__ __forceinline__ float u01(uint32_t r) {
   return fmaf(__uint2float_rn(r >> 8), 0x1p-24f, 0x1p-25f);
 }
-// ((r >> 9) + 0.5) * 2^-23, exact in binary32 and strictly inside (0, 1):
-// the Monte Carlo path's uniforms (a logarithm of each is taken)
-__device__ __forceinline__ float u01_23(uint32_t r) {
-  return fmaf(__uint2float_rn(r >> 9), 0x1p-23f, 0x1p-24f);
-}
-
 // ---------------------------------------------------------------------------
 // semianalytical histogram estimator (Sec. "Semianalytical Solution")
 //

@@ -4,13 +4,13 @@
 // compares against (Sec. "Comparison of Parametric Vs. Nonparametric
 // Models", multivariate Gaussian with Monte Carlo sampling).
 //
-// One warp per vertex.  Lanes split the samples; each sample draws two
-// Philox4x32-10 blocks (counter (s, vertex, field, j), key = seed), maps the
-// words to uniforms ((r >> 9) + 0.5) 2^-23 (exact in binary32, inside
-// (0, 1)), and Box-Muller gives six
-// normals, five of which are used.  The comparisons x_v < x_n are evaluated
-// on the differences y_n = x_v - x_n = (mu_v - mu_n) + (L_v. - L_n.) z, and
-// hits are counted with __ballot_sync + __popc.
+// One warp per vertex.  Lanes split the samples, two per turn; each sample
+// draws two Philox4x32-10 blocks (counter (s, vertex, field, j), key = seed),
+// maps the words to uniforms ((r >> 9) + 0.5) 2^-23 (exact in binary32, inside
+// (0, 1)), and Box-Muller gives six normals, five of which are used.  The
+// comparisons x_v < x_n are evaluated on the differences y_n = x_v - x_n =
+// (mu_v - mu_n) + (L_v. - L_n.) z; every lane counts its hits, and the counts
+// are added over the warp at the end.
 #include "device.cuh"
 #include "launch.h"
 
@@ -32,18 +32,35 @@ __device__ __forceinline__ void philox_pair(uint32_t s, uint32_t v, uint32_t fie
   }
 }
 
-// Box-Muller: radius sqrt(-2 ln ua), angle 2 pi ub.  The angle is taken as
-// pi + t with t = 2 pi (ub - 1/2) in [-pi, pi), where the hardware sine and
-// cosine are accurate to ~4e-7 absolute: cos(2 pi ub) = -cos t,
-// sin(2 pi ub) = -sin t.  The logarithm keeps full accuracy (its error is
-// not bounded relative to the radius near ub -> 1).
-__device__ __forceinline__ void box_muller(float ua, float ub, float &z0, float &z1) {
-  const float v = -2.f * logf(ua);
-  const float rad = v * rsqrtf(v);
-  float s, c;
-  __sincosf(6.283185307179586f * (ub - 0.5f), &s, &c);
-  z0 = -rad * c;
-  z1 = -rad * s;
+// The words of two samples (one per half) as 1 + m 2^-23, m their upper 23
+// bits: the uniforms are these minus 1 - 2^-24, exactly.
+__device__ __forceinline__ float2 word_pair(uint32_t r0, uint32_t r1) {
+  return make_float2(__uint_as_float((r0 >> 9) + 0x3f800000u),
+                     __uint_as_float((r1 >> 9) + 0x3f800000u));
+}
+
+// Box-Muller of two samples (one per half of the float2s), wa and wb their
+// words as word_pair gives them: radius sqrt(-2 ln ua), angle 2 pi ub.  The
+// angle is taken as pi + t with t = 2 pi (ub - 1/2) in [-pi, pi), where the
+// hardware sine and cosine are accurate to ~4e-7 absolute: cos(2 pi ub) = -cos
+// t, sin(2 pi ub) = -sin t.  ub - 1/2 = (wb - 3/2) + 2^-24 exactly, so one
+// multiply-add gives t with the rounding of the product.  The logarithm keeps
+// full accuracy (its error is not bounded relative to the radius near ub ->
+// 1).  Z1: also the second normal.
+template <bool Z1>
+__device__ __forceinline__ void box_muller2(float2 wa, float2 wb, float2 &z0, float2 &z1) {
+  const float c1 = -(1.f - 0x1p-24f), twopi = 6.283185307179586f;
+  const float2 ua = __fadd2_rn(wa, make_float2(c1, c1));
+  const float2 v = __fmul2_rn(make_float2(-2.f, -2.f), make_float2(logf(ua.x), logf(ua.y)));
+  const float2 rad = __fmul2_rn(v, make_float2(rsqrtf(v.x), rsqrtf(v.y)));
+  const float2 t = __ffma2_rn(__fadd2_rn(wb, make_float2(-1.5f, -1.5f)), make_float2(twopi, twopi),
+                              make_float2(twopi * 0x1p-24f, twopi * 0x1p-24f));
+  float2 sn, cs;
+  __sincosf(t.x, &sn.x, &cs.x);
+  __sincosf(t.y, &sn.y, &cs.y);
+  const float2 nr = make_float2(-rad.x, -rad.y);
+  z0 = __fmul2_rn(nr, cs);
+  if constexpr (Z1) z1 = __fmul2_rn(nr, sn);
 }
 
 // Slots of the variables: 0 = v, 1..4 = e, n, w, s.  Returns the number of
@@ -150,6 +167,66 @@ __global__ void __launch_bounds__(256) mvn_fit_kernel(Field f) {
 
 // ---------------------------------------------------------------------------
 // Monte Carlo, warp per vertex
+
+// Hits of this lane's samples (lane, lane + 32, ...): minimum and maximum, or
+// (SADDLE) the saddle in h0.  D, M: y_n = D[n] + sum_b M[n][b] z_b of the nv
+// present variables; FULL: nv = 5 (no test per neighbour).  Bound by
+// instruction issue, about 240 a sample, 35 of them 64-bit Philox products
+// (four FP32-pipe cycles each): two samples per turn, so that every FP32
+// operation but the logarithms and the special functions is a packed one (the
+// same roundings as one by one): 512 x 512 x 40, 10^4 samples 22.2 ->
+// 19.4 ms.
+template <bool SADDLE, bool FULL>
+__device__ __forceinline__ void mc_count(int S, int lane, uint32_t vid, uint32_t field,
+                                         const PhiloxKeys &K, const float *D,
+                                         const float (&M)[5][5], int nv, const float *ssg,
+                                         bool has_saddle, unsigned &h0, unsigned &h1) {
+  auto two = [&](uint32_t s0, uint32_t s1, bool second) {
+    uint4 a0, a1, b0, b1;
+    philox_pair(s0, vid, field, K, a0, a1);
+    philox_pair(s1, vid, field, K, b0, b1);
+    float2 z[6];
+    box_muller2<true>(word_pair(a0.x, b0.x), word_pair(a0.y, b0.y), z[0], z[1]);
+    box_muller2<true>(word_pair(a0.z, b0.z), word_pair(a0.w, b0.w), z[2], z[3]);
+    box_muller2<false>(word_pair(a1.x, b1.x), word_pair(a1.y, b1.y), z[4], z[5]);
+    // x_v below every neighbour: the largest y_n = x_v - x_n is < 0;
+    // above every one: the smallest is > 0
+    float2 ymax = make_float2(-kFar, -kFar), ymin = make_float2(kFar, kFar);
+    bool t1x = has_saddle, t2x = has_saddle, t1y = has_saddle, t2y = has_saddle;
+#pragma unroll
+    for (int n = 1; n < 5; ++n) {
+      if (FULL || n < nv) {
+        float2 yv = make_float2(D[n], D[n]);
+#pragma unroll
+        for (int b = 0; b <= n; ++b) yv = __ffma2_rn(make_float2(M[n][b], M[n][b]), z[b], yv);
+        if constexpr (SADDLE) {
+          // t1 wants x_v < x_n where the sign is +1
+          const float sx = ssg[n] * yv.x, sy = ssg[n] * yv.y;
+          t1x &= sx < 0.f;
+          t2x &= sx > 0.f;
+          t1y &= sy < 0.f;
+          t2y &= sy > 0.f;
+        } else {
+          ymax = make_float2(fmaxf(ymax.x, yv.x), fmaxf(ymax.y, yv.y));
+          ymin = make_float2(fminf(ymin.x, yv.x), fminf(ymin.y, yv.y));
+        }
+      }
+    }
+    if constexpr (SADDLE) {
+      h0 += (t1x || t2x) ? 1u : 0u;
+      h0 += (second && (t1y || t2y)) ? 1u : 0u;
+    } else {
+      h0 += ymax.x < 0.f ? 1u : 0u;
+      h1 += ymin.x > 0.f ? 1u : 0u;
+      h0 += (second && ymax.y < 0.f) ? 1u : 0u;
+      h1 += (second && ymin.y > 0.f) ? 1u : 0u;
+    }
+  };
+  const uint32_t whole = (uint32_t)S & ~63u;
+  for (uint32_t s = 0; s < whole; s += 64) two(s + lane, s + 32 + lane, true);
+  const uint32_t s = whole + lane;
+  if (s < (uint32_t)S) two(s, s + 32, s + 32 < (uint32_t)S);
+}
 
 template <bool FROM_MEMBERS, bool SADDLE>
 __global__ void __launch_bounds__(256) mvn_mc_kernel(Field f, int S, uint32_t k0, uint32_t k1,
@@ -293,46 +370,14 @@ __global__ void __launch_bounds__(256) mvn_mc_kernel(Field f, int S, uint32_t k0
 #pragma unroll
           for (int b = 0; b < 5; ++b) M[n][b] = (b == 0 ? L[0][0] : 0.f) - L[n][b];
         }
-        unsigned cmin = 0, cmax = 0, csad = 0;
-        const int iters = (S + 31) >> 5;
-        const uint32_t vid = (uint32_t)v;
+        unsigned h0 = 0, h1 = 0;
         const PhiloxKeys K(k0, k1);
-        for (int it = 0; it < iters; ++it) {
-          const int s = (it << 5) + lane;
-          uint4 r0, r1;
-          philox_pair((uint32_t)s, vid, field, K, r0, r1);
-          float z[6];
-          box_muller(u01_23(r0.x), u01_23(r0.y), z[0], z[1]);
-          box_muller(u01_23(r0.z), u01_23(r0.w), z[2], z[3]);
-          box_muller(u01_23(r1.x), u01_23(r1.y), z[4], z[5]);
-          // x_v below every neighbour: the largest y_n = x_v - x_n is < 0;
-          // above every one: the smallest is > 0
-          float ymax = -kFar, ymin = kFar;
-          bool t1 = has_saddle, t2 = has_saddle;
-#pragma unroll
-          for (int n = 1; n < 5; ++n) {
-            if (n < nv) {
-              float yv = D[n];
-#pragma unroll
-              for (int b = 0; b <= n; ++b) yv = fmaf(M[n][b], z[b], yv);
-              ymax = fmaxf(ymax, yv);
-              ymin = fminf(ymin, yv);
-              if constexpr (SADDLE) {
-                // y = x_v - x_n: t1 wants x_v < x_n where the sign is +1
-                const float sy = ssg[n] * yv;
-                t1 &= sy < 0.f;
-                t2 &= sy > 0.f;
-              }
-            }
-          }
-          const bool valid = s < S;
-          if constexpr (!SADDLE) {
-            cmin += __popc(__ballot_sync(0xffffffffu, valid && ymax < 0.f));
-            cmax += __popc(__ballot_sync(0xffffffffu, valid && ymin > 0.f));
-          } else {
-            csad += __popc(__ballot_sync(0xffffffffu, valid && (t1 || t2)));
-          }
-        }
+        if (nv == 5)
+          mc_count<SADDLE, true>(S, lane, (uint32_t)v, field, K, D, M, nv, ssg, has_saddle, h0, h1);
+        else
+          mc_count<SADDLE, false>(S, lane, (uint32_t)v, field, K, D, M, nv, ssg, has_saddle, h0, h1);
+        const unsigned cmin = __reduce_add_sync(0xffffffffu, h0), csad = cmin;
+        const unsigned cmax = __reduce_add_sync(0xffffffffu, h1);
         pmin = zero_mm ? 0.f : (float)cmin / (float)S;
         pmax = zero_mm ? 0.f : (float)cmax / (float)S;
         psad = (float)csad / (float)S;
