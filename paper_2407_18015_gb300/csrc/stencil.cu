@@ -220,8 +220,14 @@ __global__ void __launch_bounds__(NTHREADS, 2) stencil_hist_kernel(StencilField 
     }
     if (z < 0 || z >= f.D || y < 0 || y >= f.H || x < 0 || x >= f.W) continue;
     HistParamRegs<RB> P;
-    P.load(pf, z * HW + (long long)y * f.W + x, B, false);
-    hist_rows_build_regs<SLOTS, RS, RB>(P, sm, R4, l, B);
+    const long long gi = z * HW + (long long)y * f.W + x;
+    if (B == RB) {
+      P.template load<true>(pf, gi, B, false);
+      hist_rows_build_regs<SLOTS, RS, RB, true>(P, sm, R4, l, B);
+    } else {
+      P.template load<false>(pf, gi, B, false);
+      hist_rows_build_regs<SLOTS, RS, RB, false>(P, sm, R4, l, B);
+    }
   }
   __syncthreads();
   const int v = threadIdx.x, vx = v & 31;

@@ -361,26 +361,39 @@ __device__ __forceinline__ void hist_tail_table(float *sm, int l, int B) {
 
 // Per-bin rows of one vertex (see hist_r4_rows) from its lo, hi and masses
 // m_0..m_{B-1} (all FP32): R[k * RS] for k = 0..B.  T = m_0 + ... + m_{B-1}
-// in bin order; the tails S_k = T - (m_0 + ... + m_{k-1}).
-template <int RS, typename Mass>
-__device__ __forceinline__ void hist_rows_build(float4 *R, float a, float b, float t, int B,
+// in bin order; the tails S_k = T - (m_0 + ... + m_{k-1}).  NB: the number of
+// bins if it is known at compile time (no test per bin, constant edges), else
+// the bound that the loop is unrolled to (0: not unrolled).  ADJ (the adjoint,
+// which walks the survivals alone): the second entry of a row is 1 / h on a
+// bin and 0 beyond the support instead of T - S_k.
+template <int RS, int NB, bool FULL, bool ADJ = false, typename Mass>
+__device__ __forceinline__ void hist_rows_write(float4 *R, float a, float b, float t, int B,
                                                 Mass mass) {
-  const float4 beyond = make_float4(0.f, t, 0.f, kFar);
+  if constexpr (FULL) B = NB;
+  const float4 beyond = make_float4(0.f, ADJ ? 0.f : t, 0.f, kFar);
+  R[B * RS] = beyond;
   if (a == b) {
-    for (int k = 0; k < hist_r4_rows(B); ++k) R[k * RS] = beyond;
+    for (int k = 0; k < B; ++k) R[k * RS] = beyond;
     return;
   }
   // for a power of two B the product with 1/B is the quotient exactly
   const float w = b - a;
   const float h = (B & (B - 1)) == 0 ? w * (1.f / (float)B) : w / (float)B, ih = frcp(h);
   float c = 0.f, sk = t;
-  for (int k = 0; k < B; ++k) {
+  auto row = [&](int k) {
     c += mass(k);
     const float sn = k + 1 < B ? t - c : 0.f;
-    R[k * RS] = make_float4(sk, t - sk, (sk - sn) * ih, k + 1 < B ? (float)(k + 1) * h : w);
+    R[k * RS] = make_float4(sk, ADJ ? ih : t - sk, (sk - sn) * ih,
+                            k + 1 < B ? (float)(k + 1) * h : w);
     sk = sn;
+  };
+  if constexpr (NB > 0) {
+#pragma unroll
+    for (int k = 0; k < NB; ++k)
+      if (FULL || k < B) row(k);
+  } else {
+    for (int k = 0; k < B; ++k) row(k);
   }
-  R[B * RS] = beyond;
 }
 
 // Per-bin rows of staged vertex l from the masses in its parameter tile
@@ -398,119 +411,95 @@ __device__ __forceinline__ void hist_row_table(float *sm, float4 *R, int l, int 
     else if (w < 0.f) st |= V_BAD;
     t += w;
   }
-  hist_rows_build<RS>(R + l, a, b, t, B, [&](int k) { return sm[(2 + k) * HALO + l]; });
+  hist_rows_write<RS, 0, false>(R + l, a, b, t, B,
+                                [&](int k) { return sm[(2 + k) * HALO + l]; });
   sm[2 * HALO + l] = t;
   sm[3 * HALO + l] = (float)st;
 }
 
 // The same from bin counts kept in registers (fitted mass count / N of bin k
 // from cnt_mass(k)), for a vertex fitted from its members: lo = mn, hi = mx;
-// nf marks non-finite members (all parameters NaN), mn == mx a point mass
-// (mass 1 in bin 0).  The same masses, total, rows and status as the
+// nf marks non-finite members (no rows: no walk reads them), mn == mx a point
+// mass (mass 1 in bin 0).  The same masses, total, rows and status as the
 // parameter tile and hist_row_table give.
+template <int HALO, int RS, int RB, bool FULL, typename Mass>
+__device__ __forceinline__ void hist_row_table_counts_n(float *sm, float4 *R, int l, int B,
+                                                        bool nf, float mn, float mx,
+                                                        Mass cnt_mass) {
+  if constexpr (FULL) B = RB;
+  float m[RB];
+  float t = nf ? qnan() : 1.f;
+  if (!nf && mn != mx) {
+    t = 0.f;
+#pragma unroll
+    for (int q = 0; q < RB; ++q)
+      if (FULL || q < B) {
+        m[q] = cnt_mass(q);
+        t += m[q];
+      }
+  }
+  if (!nf) hist_rows_write<RS, RB, FULL>(R + l, mn, mx, t, B, [&](int k) { return m[k]; });
+  sm[2 * HALO + l] = t;
+  sm[3 * HALO + l] = (float)(nf ? V_NONFINITE : (mn == mx ? V_DEGENERATE : 0));
+}
 template <int HALO, int RS, int RB, typename Mass>
 __device__ __forceinline__ void hist_row_table_counts(float *sm, float4 *R, int l, int B, bool nf,
                                                       float mn, float mx, Mass cnt_mass) {
-  // at most RB bins: every loop unrolled to RB with the bins past B idle
-  float m[RB];
-  float t = 0.f;
-#pragma unroll
-  for (int q = 0; q < RB; ++q) {
-    m[q] = 0.f;
-    if (q < B) {
-      m[q] = nf ? qnan() : (mn == mx ? (q == 0 ? 1.f : 0.f) : cnt_mass(q));
-      t += m[q];
-    }
-  }
-  const uint8_t st = nf ? V_NONFINITE : (mn == mx ? V_DEGENERATE : 0);
-  R += l;
-  const float a = nf ? qnan() : mn, b = nf ? qnan() : mx;
-  const float4 beyond = make_float4(0.f, t, 0.f, kFar);
-  if (a == b) {
-#pragma unroll
-    for (int k = 0; k <= RB; ++k)
-      if (k <= B) R[k * RS] = beyond;
-  } else {
-    // as hist_rows_build
-    const float w = b - a;
-    const float h = (B & (B - 1)) == 0 ? w * (1.f / (float)B) : w / (float)B, ih = frcp(h);
-    float c = 0.f, sk = t;
-#pragma unroll
-    for (int k = 0; k < RB; ++k) {
-      if (k < B) {
-        c += m[k];
-        const float sn = k + 1 < B ? t - c : 0.f;
-        R[k * RS] = make_float4(sk, t - sk, (sk - sn) * ih, k + 1 < B ? (float)(k + 1) * h : w);
-        sk = sn;
-      }
-    }
-    R[B * RS] = beyond;
-  }
-  sm[2 * HALO + l] = t;
-  sm[3 * HALO + l] = (float)st;
+  if (B == RB) hist_row_table_counts_n<HALO, RS, RB, true>(sm, R, l, B, nf, mn, mx, cnt_mass);
+  else hist_row_table_counts_n<HALO, RS, RB, false>(sm, R, l, B, nf, mn, mx, cnt_mass);
 }
 
 // The parameters of one vertex in registers (mirrored: -X, bins
 // reversed): support [a, b] and masses m[0..B-1], read with every load in
-// flight at once.
+// flight at once.  FULL: B is the compile-time RB.
 template <int RB>
 struct HistParamRegs {
   float a, b, m[RB];
+  template <bool FULL>
   __device__ __forceinline__ void load(const Field &f, long long gi, int B, bool mirrored) {
+    if constexpr (FULL) B = RB;
     const long long plane = f.plane;
-    const float a0 = __ldg(f.params + gi), b0 = __ldg(f.params + plane + gi);
+    const float *p = f.params + gi;
+    const float a0 = __ldg(p), b0 = __ldg(p + plane);
     a = mirrored ? -b0 : a0;
     b = mirrored ? -a0 : b0;
+    const float *q0 = p + (mirrored ? (long long)(1 + B) * plane : 2 * plane);
+    const long long step = mirrored ? -plane : plane;
 #pragma unroll
-    for (int q = 0; q < RB; ++q)
-      m[q] = q < B ? __ldg(f.params + (long long)(2 + (mirrored ? B - 1 - q : q)) * plane + gi)
-                   : 0.f;
+    for (int q = 0; q < RB; ++q) m[q] = FULL || q < B ? __ldg(q0 + q * step) : 0.f;
   }
 };
 
 // Per-bin rows, lo, hi, total and status of one staged vertex from its
 // parameters in registers; the same rows and status as hist_row_table
-// builds from a parameter tile.  ADJ (the adjoint, which walks the survivals
-// alone): the second entry of a row is 1 / h on a bin and 0 beyond the
-// support instead of T - S_k.
-template <int HALO, int RS, int RB, bool ADJ = false>
+// builds from a parameter tile (ADJ: see hist_rows_write).
+template <int HALO, int RS, int RB, bool FULL, bool ADJ = false>
 __device__ __forceinline__ void hist_rows_build_regs(const HistParamRegs<RB> &P, float *sm,
                                                      float4 *R, int l, int B) {
+  if constexpr (FULL) B = RB;
   const float a = P.a, b = P.b;
   uint8_t st = (!isfinite(a) || !isfinite(b)) ? V_NONFINITE
                                              : (a > b ? V_BAD : (a == b ? V_DEGENERATE : 0));
-  float t = 0.f;
+  // smallest and largest mass (NaN-propagating): a finite smallest and
+  // largest mean that all are finite, and its sign says the rest; the slots
+  // past B hold 0
+  float t = 0.f, mn = P.m[0], mx = P.m[0];
 #pragma unroll
   for (int q = 0; q < RB; ++q) {
-    if (q < B) {
+    if (FULL || q < B) t += P.m[q];
+    mn = fmin_nan(mn, P.m[q]);
+    mx = fmax_nan(mx, P.m[q]);
+  }
+  if (isfinite(mn) && isfinite(mx)) {
+    if (mn < 0.f) st |= V_BAD;
+  } else {
+#pragma unroll
+    for (int q = 0; q < RB; ++q) {
       if (!isfinite(P.m[q])) st |= V_NONFINITE;
       else if (P.m[q] < 0.f) st |= V_BAD;
-      t += P.m[q];
     }
   }
-  R += l;
-  const float4 beyond = make_float4(0.f, ADJ ? 0.f : t, 0.f, kFar);
-  if (a == b) {
-#pragma unroll
-    for (int k = 0; k <= RB; ++k)
-      if (k <= B) R[k * RS] = beyond;
-  } else {
-    // as hist_rows_build
-    const float w = b - a;
-    const float h = (B & (B - 1)) == 0 ? w * (1.f / (float)B) : w / (float)B, ih = frcp(h);
-    float c = 0.f, sk = t;
-#pragma unroll
-    for (int k = 0; k < RB; ++k) {
-      if (k < B) {
-        c += P.m[k];
-        const float sn = k + 1 < B ? t - c : 0.f;
-        R[k * RS] = make_float4(sk, ADJ ? ih : t - sk, (sk - sn) * ih,
-                                k + 1 < B ? (float)(k + 1) * h : w);
-        sk = sn;
-      }
-    }
-    R[B * RS] = beyond;
-  }
+  hist_rows_write<RS, RB, FULL, ADJ>(R + l, a, b, t, B, [&](int k) { return P.m[k]; });
   sm[l] = a;
   sm[HALO + l] = b;
   sm[2 * HALO + l] = t;
@@ -521,39 +510,42 @@ __device__ __forceinline__ void hist_rows_build_regs(const HistParamRegs<RB> &P,
 // the parameters.  BATCH: each thread first reads the parameters of all the
 // halo vertices it owns (l = tid, tid + NTHREADS, ...), every load in
 // flight at once, then builds their rows -- for kernels at two CTAs per SM,
-// whose CTA otherwise waits for two rounds of reads (2048 x 2048 x 50, 16
-// bins: forward from parameters 1.11 -> 1.06 ms, adjoint 2.85 -> 2.83 ms);
-// else one vertex after another (the 8-bin forward at four CTAs per SM:
-// 0.53 ms, against 0.57 batched).
+// whose CTA otherwise waits for two rounds of reads; else one vertex after
+// another.  With the bins known at compile time (B = RB: 8 and 16) a vertex
+// has no test per bin: 2048 x 2048 vertices, 16 bins, fit + forward +
+// adjoint 3.62 -> 3.51 ms.
+template <int HALO, int RS, int RB, int HX, bool BATCH, bool ADJ, bool FULL>
+__device__ __forceinline__ void hist_rows_from_params_n(const Field &f, float *sm, float4 *R,
+                                                        int ty0, int tx0, int ylim, int B,
+                                                        bool mirrored) {
+  constexpr int PER = BATCH ? (HALO + NTHREADS - 1) / NTHREADS : 1;
+  HistParamRegs<RB> P[PER];
+  bool in[PER];
+  for (int l0 = threadIdx.x; l0 < HALO; l0 += PER * NTHREADS) {
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
+      const int l = l0 + p * NTHREADS;
+      const int r = l / HX, c = l - r * HX;
+      const int gy = ty0 + r - 1, gx = tx0 + c - 1;
+      in[p] = l < HALO && gy >= 0 && gy < ylim && gx >= 0 && gx < f.W;
+      if (in[p]) P[p].template load<FULL>(f, (long long)gy * f.W + gx, B, mirrored);
+    }
+#pragma unroll
+    for (int p = 0; p < PER; ++p)
+      if (in[p])
+        hist_rows_build_regs<HALO, RS, RB, FULL, ADJ>(P[p], sm, R, l0 + p * NTHREADS, B);
+  }
+}
 template <int HALO, int RS, int RB, int HX, bool BATCH, bool ADJ = false>
 __device__ __forceinline__ void hist_rows_from_params_tile(const Field &f, float *sm, float4 *R,
                                                            int ty0, int tx0, int ylim, int B,
                                                            bool mirrored) {
-  if constexpr (!BATCH) {
-    for (int l = threadIdx.x; l < HALO; l += NTHREADS) {
-      const int r = l / HX, c = l - r * HX;
-      const int gy = ty0 + r - 1, gx = tx0 + c - 1;
-      if (gy < 0 || gy >= ylim || gx < 0 || gx >= f.W) continue;
-      HistParamRegs<RB> P;
-      P.load(f, (long long)gy * f.W + gx, B, mirrored);
-      hist_rows_build_regs<HALO, RS, RB, ADJ>(P, sm, R, l, B);
-    }
-    return;
-  }
-  constexpr int PER = (HALO + NTHREADS - 1) / NTHREADS;
-  HistParamRegs<RB> P[PER];
-  bool in[PER];
-#pragma unroll
-  for (int p = 0; p < PER; ++p) {
-    const int l = threadIdx.x + p * NTHREADS;
-    const int r = l / HX, c = l - r * HX;
-    const int gy = ty0 + r - 1, gx = tx0 + c - 1;
-    in[p] = l < HALO && gy >= 0 && gy < ylim && gx >= 0 && gx < f.W;
-    if (in[p]) P[p].load(f, (long long)gy * f.W + gx, B, mirrored);
-  }
-#pragma unroll
-  for (int p = 0; p < PER; ++p)
-    if (in[p]) hist_rows_build_regs<HALO, RS, RB, ADJ>(P[p], sm, R, threadIdx.x + p * NTHREADS, B);
+  if (B == RB)
+    hist_rows_from_params_n<HALO, RS, RB, HX, BATCH, ADJ, true>(f, sm, R, ty0, tx0, ylim, B,
+                                                                mirrored);
+  else
+    hist_rows_from_params_n<HALO, RS, RB, HX, BATCH, ADJ, false>(f, sm, R, ty0, tx0, ylim, B,
+                                                                 mirrored);
 }
 
 // ---------------------------------------------------------------------------
