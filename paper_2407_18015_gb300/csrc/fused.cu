@@ -28,6 +28,7 @@ namespace {
 
 constexpr int kTY3 = 8, kHALO3 = (kTY3 + 2) * 34, kRS3 = hist_r4_stride(kHALO3);
 constexpr int kOcc3 = 3;  // resident CTAs per SM
+constexpr int kSplitCtas = 152;  // one CTA per SM
 
 // Shared memory of a fused tile, in floats: the member box, whose room the
 // histogram's per-bin rows take after the last read of the box; the
@@ -43,11 +44,13 @@ __host__ __device__ constexpr long long etile3_floats() { return 2LL * kHALO3; }
 // Staging of one fused tile (see stage_members_tma: the same box walk, the
 // same per-vertex arithmetic for each model; ASYNC: the box filled by
 // asynchronous copies, members the tensor memory accelerator cannot
-// address).  Returns false if a bounded wait gave up.
-template <bool ASYNC>
+// address).  SPLIT: what model `only` needs alone.  Returns false if a bounded
+// wait gave up.
+template <bool ASYNC, bool SPLIT>
 __device__ __forceinline__ bool stage3(const Field &f, float *smh, float *sme, float *box,
                                        uint64_t *bar, const CUtensorMap *tmap, int ty0, int tx0,
-                                       float4 *R4) {
+                                       float4 *R4, int only) {
+  const bool epan = !SPLIT || only == 1;
   constexpr int HY = kTY3 + 2, HX = 34, HALO = kHALO3;
   constexpr int PER = (HALO + NTHREADS - 1) / NTHREADS;
   constexpr int PLANE = HY * kBoxW;
@@ -117,34 +120,28 @@ __device__ __forceinline__ bool stage3(const Field &f, float *smh, float *sme, f
       if (!in[p]) continue;
       const int sh = shift0(p, k0);
       const float *col = box + off[p] + sh;
-      // member k of the box at col[at(k)]
-      auto at = [&](int k) { return k * PLANE + (pl == 0 ? 0 : ((sh + k * pl) & 3) - sh); };
       // as stage_members_tma: member 0 starts min / max (and adds 0 to the
-      // sums), the others in pairs into NaN-propagating min / max
-      int k = 0;
-      if (k0 == 0) {
-        x0[p] = mn[p] = mx[p] = col[0];
-        k = 1;
-      }
+      // sums), members go in pairs into NaN-propagating min / max
+      if (k0 == 0) x0[p] = mn[p] = mx[p] = col[0];
       auto add = [&](float v) {
         const float d = v - x0[p];
         s1[p].add(d);
         s2[p].add(d * d);
       };
-#pragma unroll 4
-      for (; k + 1 < kn; k += 2) {
-        const float v1 = col[at(k)], v2 = col[at(k + 1)];
-        mn[p] = fmin3_nan(mn[p], v1, v2);
-        mx[p] = fmax3_nan(mx[p], v1, v2);
-        add(v1);
-        add(v2);
-      }
-      if (k < kn) {
-        const float v = col[at(k)];
-        mn[p] = fmin_nan(mn[p], v);
-        mx[p] = fmax_nan(mx[p], v);
-        add(v);
-      }
+      box_members<PLANE, ASYNC>(col, kn, sh, pl, MemberPairs{
+          [&](float v1, float v2) {
+            mn[p] = fmin3_nan(mn[p], v1, v2);
+            mx[p] = fmax3_nan(mx[p], v1, v2);
+            if (epan) {
+              add(v1);
+              add(v2);
+            }
+          },
+          [&](float v) {
+            mn[p] = fmin_nan(mn[p], v);
+            mx[p] = fmax_nan(mx[p], v);
+            if (epan) add(v);
+          }});
     }
     __syncthreads();
   }
@@ -169,6 +166,7 @@ __device__ __forceinline__ bool stage3(const Field &f, float *smh, float *sme, f
     sme[l] = nf[p] ? qnan() : m;
     sme[HALO + l] = nf[p] ? qnan() : w;
   }
+  if (SPLIT && only != 2) return true;
   // pass 2 (boxes in reverse: the last one of pass 1 is still there): bin
   // counts, 8-bit counters packed in a 64-bit word for up to 255 members,
   // 16-bit ones in two words for more
@@ -195,14 +193,20 @@ __device__ __forceinline__ bool stage3(const Field &f, float *smh, float *sme, f
         if (!bin[p]) continue;
         const int sh = shift0(p, k0);
         const float *col = box + off[p] + sh;
-        auto at = [&](int k) { return k * PLANE + (pl == 0 ? 0 : ((sh + k * pl) & 3) - sh); };
+        auto count8 = [&](float v) {
+          cw[p][0] += 1ull << (hist_bin_nonneg(v, mn[p], sc[p], B) << 3);
+        };
         if (!wide) {
-#pragma unroll 4
-          for (int k = 0; k < kn; ++k)
-            cw[p][0] += 1ull << (hist_bin_nonneg(col[at(k)], mn[p], sc[p], B) << 3);
+          box_members<PLANE, ASYNC>(col, kn, sh, pl, MemberPairs{
+              [&](float v1, float v2) {
+                count8(v1);
+                count8(v2);
+              },
+              count8});
         } else {
           for (int k = 0; k < kn; ++k) {
-            const int j = hist_bin_nonneg(col[at(k)], mn[p], sc[p], B);
+            const int j =
+                hist_bin_nonneg(col[k * PLANE + (((sh + k * pl) & 3) - sh)], mn[p], sc[p], B);
             const unsigned long long inc = 1ull << ((j & 3) << 4);
             cw[p][0] += (j >> 2) == 0 ? inc : 0ull;
             cw[p][1] += (j >> 2) == 1 ? inc : 0ull;
@@ -227,9 +231,10 @@ __device__ __forceinline__ bool stage3(const Field &f, float *smh, float *sme, f
 }
 
 // Every vertex of a staged fused tile under the three models (the uniform,
-// Epanechnikov and histogram branches of integrate_tile).
+// Epanechnikov and histogram branches of integrate_tile); SPLIT: model `only`.
+template <bool SPLIT>
 __device__ __forceinline__ void integrate3(const Field3 &F, int ty0, int tx0, const float *smh,
-                                           const float *sme, const float4 *R4) {
+                                           const float *sme, const float4 *R4, int only) {
   constexpr int TX = 32, HX = 34, HALO = kHALO3, RS = kRS3;
   const Field &f = F.f;
   const int B = f.B;
@@ -256,7 +261,7 @@ __device__ __forceinline__ void integrate3(const Field3 &F, int ty0, int tx0, co
     if (F.status[m]) F.status[m][gi] = st;
   };
   // uniform (parameters: the histogram tile's lo, hi)
-  {
+  if (!SPLIT || only == 0) {
     float T[4], Tc;
     uint8_t st = check_params<kUniform, HALO>(smh, l, B, Tc);
 #pragma unroll
@@ -276,7 +281,7 @@ __device__ __forceinline__ void integrate3(const Field3 &F, int ty0, int tx0, co
     put(0, pmin, pmax, st);
   }
   // Epanechnikov
-  {
+  if (!SPLIT || only == 1) {
     float T[4], Tc;
     uint8_t st = check_params<kEpan, HALO>(sme, l, B, Tc);
 #pragma unroll
@@ -296,7 +301,7 @@ __device__ __forceinline__ void integrate3(const Field3 &F, int ty0, int tx0, co
     put(1, pmin, pmax, st);
   }
   // histogram: the per-bin row walk
-  {
+  if (!SPLIT || only == 2) {
     float T[4], Tc;
     uint8_t st = check_params<kHist, HALO, true>(smh, l, B, Tc);
 #pragma unroll
@@ -342,7 +347,7 @@ __device__ __forceinline__ void integrate3(const Field3 &F, int ty0, int tx0, co
   }
 }
 
-template <bool ASYNC>
+template <bool ASYNC, bool SPLIT>
 __global__ void __launch_bounds__(NTHREADS, kOcc3)
     tile3_kernel(Field3 F, int tiles_x, const __grid_constant__ CUtensorMap tmap) {
   extern __shared__ __align__(128) float smem[];
@@ -354,13 +359,15 @@ __global__ void __launch_bounds__(NTHREADS, kOcc3)
   float *sme = smh + htile3_floats();
   uint64_t *bar = reinterpret_cast<uint64_t *>(sme + ((etile3_floats() + 1) & ~1LL));
   float4 *R4 = reinterpret_cast<float4 *>(smem);
-  const bool ok = stage3<ASYNC>(f, smh, sme, smem, bar, &tmap, ty0, tx0, R4);
+  const int only = SPLIT ? (int)blockIdx.y : -1;  // one model per row of CTAs
+  const bool ok = stage3<ASYNC, SPLIT>(f, smh, sme, smem, bar, &tmap, ty0, tx0, R4, only);
   __syncthreads();
   if (!ok) {  // a bounded wait gave up: NaN and the timeout flag, every model
     const int v = threadIdx.x, gy = ty0 + v / 32, gx = tx0 + v % 32;
     if (gy < f.y1 && gx < f.W) {
       const long long gi = (long long)gy * f.W + gx;
       for (int m = 0; m < 3; ++m) {
+        if (SPLIT && m != only) continue;
         if ((f.cptypes & kMin) && F.out_min[m]) F.out_min[m][gi] = qnan();
         if ((f.cptypes & kMax) && F.out_max[m]) F.out_max[m][gi] = qnan();
         if (F.status[m]) F.status[m][gi] = V_TIMEOUT;
@@ -368,7 +375,7 @@ __global__ void __launch_bounds__(NTHREADS, kOcc3)
     }
     return;
   }
-  integrate3(F, ty0, tx0, smh, sme, R4);
+  integrate3<SPLIT>(F, ty0, tx0, smh, sme, R4, only);
 }
 
 }  // namespace
@@ -417,11 +424,10 @@ cudaError_t launch_closed3(const Field3 &F, cudaStream_t s, bool *launched) {
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 128) return cudaErrorInvalidDevice;
   if (!attr_set[dev].load(std::memory_order_acquire)) {
-    e = cudaFuncSetAttribute(tile3_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             227 * 1024);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(tile3_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               227 * 1024);
+    for (auto k : {tile3_kernel<false, false>, tile3_kernel<true, false>,
+                   tile3_kernel<false, true>, tile3_kernel<true, true>})
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) {
       cudaGetLastError();
       return e;
@@ -431,10 +437,16 @@ cudaError_t launch_closed3(const Field3 &F, cudaStream_t s, bool *launched) {
   Field3 G = F;
   G.f.tma_nc = nc;
   const size_t smem = std::max((size_t)nc * per_member, rows_b) + fixed_b;
-  if (tma)
-    tile3_kernel<false><<<(int)tiles, NTHREADS, smem, s>>>(G, tiles_x, map);
-  else
-    tile3_kernel<true><<<(int)tiles, NTHREADS, smem, s>>>(G, tiles_x, map);
+  // A grid whose tiles leave SMs empty even three times over (up to 50 tiles
+  // of 8 x 32: a 64 x 64 field has 16) takes three CTAs per tile, one per
+  // model: each then waits for one model's chain of stages and not for the
+  // sum of the three, and staging a tile three times costs nothing there
+  // (64 x 64 x 20: 13.1 -> 10.9 us a
+  // launch, launch included; 128 x 128 x 20, 64 tiles: 13.4 -> 15.1)
+  const bool split = tiles * 3 <= kSplitCtas;
+  auto k = split ? (tma ? tile3_kernel<false, true> : tile3_kernel<true, true>)
+                 : (tma ? tile3_kernel<false, false> : tile3_kernel<true, false>);
+  k<<<dim3((unsigned)tiles, split ? 3u : 1u), NTHREADS, smem, s>>>(G, tiles_x, map);
   *launched = true;
   return cudaGetLastError();
 }

@@ -645,6 +645,47 @@ __device__ __forceinline__ void box_copy_async(const Field &f, float *box, int k
   __syncthreads();
 }
 
+// two callables as one: on a pair of members and on a single one
+template <typename F2, typename F1>
+struct MemberPairs {
+  F2 two;
+  F1 one;
+  __device__ __forceinline__ void operator()(float a, float b) const { two(a, b); }
+  __device__ __forceinline__ void operator()(float a) const { one(a); }
+};
+template <typename F2, typename F1>
+__device__ MemberPairs(F2, F1) -> MemberPairs<F2, F1>;
+
+// f(v) for the members 0 .. kn-1 of a box at one column, in order: member k
+// is at col[k * PLANE + o], o = ((sh + k pl) & 3) - sh the element shift of
+// asynchronously copied members relative to member 0's (0 for the tensor
+// memory accelerator), which repeats every four members: four to a turn, so
+// that the shifts are formed once per box and not per read.
+template <int PLANE, bool ASYNC, typename F>
+__device__ __forceinline__ void box_members(const float *col, int kn, int sh, int pl, F f) {
+  const float *c1 = col + PLANE, *c2 = col + 2 * PLANE, *c3 = col + 3 * PLANE;
+  if constexpr (ASYNC) {
+    c1 += ((sh + pl) & 3) - sh;
+    c2 += ((sh + 2 * pl) & 3) - sh;
+    c3 += ((sh + 3 * pl) & 3) - sh;
+  }
+  // turns unrolled: 1021 x 1023 x 50, 5 bins, asynchronous copies 184 (before)
+  // -> 180, 178, 176 us with one, two, four turns; 1024 x 1024 x 20, three
+  // models, tensor memory accelerator 207, 209, 213 us
+  constexpr int kTurns = ASYNC ? 4 : 1;
+  int k = 0;
+#pragma unroll kTurns
+  for (; k + 4 <= kn; k += 4) {
+    const float v[4] = {col[k * PLANE], c1[k * PLANE], c2[k * PLANE], c3[k * PLANE]};
+    f(v[0], v[1]);
+    f(v[2], v[3]);
+  }
+  // up to three more
+  if (k + 1 < kn) f(col[k * PLANE], c1[k * PLANE]);
+  if (k + 2 < kn) f(c2[k * PLANE]);
+  else if (k < kn && k + 1 == kn) f(col[k * PLANE]);
+}
+
 // wait for the completion of phase `parity`; gives up after a bounded number
 // of polls (each poll itself returns after a bounded time)
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity) {
@@ -777,14 +818,10 @@ __device__ __forceinline__ bool stage_members_tma(const Field &f, float *sm, flo
       const int sh = shift0(p, k0);
       const float *col = box + off[p] + sh;
       // member 0 starts the running min / max (and is the shift x0 of the
-      // Epanechnikov sums, to which it adds 0); the others go in pairs into
+      // Epanechnikov sums, to which it adds 0); members go in pairs into
       // NaN-propagating three-input min / max, so that a non-finite member
       // shows in mn / mx (nf below)
-      int k = 0;
-      if (k0 == 0) {
-        x0[p] = mn[p] = mx[p] = col[0];
-        k = 1;
-      }
+      if (k0 == 0) x0[p] = mn[p] = mx[p] = col[0];
       auto add = [&](float v) {
         if constexpr (EP) {
           const float d = v - x0[p];
@@ -792,26 +829,18 @@ __device__ __forceinline__ bool stage_members_tma(const Field &f, float *sm, flo
           s2[p].add(d * d);
         }
       };
-      auto add2 = [&](float v1, float v2) {
-        mn[p] = fmin3_nan(mn[p], v1, v2);
-        mx[p] = fmax3_nan(mx[p], v1, v2);
-        add(v1);
-        add(v2);
-      };
-      if (pl == 0) {
-#pragma unroll 4
-        for (; k + 1 < kn; k += 2) add2(col[k * PLANE], col[(k + 1) * PLANE]);
-      } else {
-        for (; k + 1 < kn; k += 2)
-          add2(col[k * PLANE + (((sh + k * pl) & 3) - sh)],
-               col[(k + 1) * PLANE + (((sh + (k + 1) * pl) & 3) - sh)]);
-      }
-      if (k < kn) {
-        const float v = col[k * PLANE + (((sh + k * pl) & 3) - sh)];
-        mn[p] = fmin_nan(mn[p], v);
-        mx[p] = fmax_nan(mx[p], v);
-        add(v);
-      }
+      box_members<PLANE, ASYNC>(col, kn, sh, pl, MemberPairs{
+          [&](float v1, float v2) {
+            mn[p] = fmin3_nan(mn[p], v1, v2);
+            mx[p] = fmax3_nan(mx[p], v1, v2);
+            add(v1);
+            add(v2);
+          },
+          [&](float v) {
+            mn[p] = fmin_nan(mn[p], v);
+            mx[p] = fmax_nan(mx[p], v);
+            add(v);
+          }});
     }
     __syncthreads();
   }
@@ -906,18 +935,15 @@ __device__ __forceinline__ bool stage_members_tma(const Field &f, float *sm, flo
 #pragma unroll
             for (int w = 0; w < NW16; ++w) cw[p][w] += (j >> 2) == w ? inc : 0ull;
           };
-          if (pl != 0) {
-            for (int k = 0; k < kn; ++k) {
-              const float v = col[k * PLANE + (((sh + k * pl) & 3) - sh)];
-              if (!wide) count8(v);
-              else count16(v);
-            }
-          } else if (!wide) {
-#pragma unroll 4
-            for (int k = 0; k < kn; ++k) count8(col[k * PLANE]);
-          } else {
-            for (int k = 0; k < kn; ++k) count16(col[k * PLANE]);
-          }
+          if (!wide)
+            box_members<PLANE, ASYNC>(col, kn, sh, pl, MemberPairs{
+                [&](float v1, float v2) {
+                  count8(v1);
+                  count8(v2);
+                },
+                count8});
+          else
+            for (int k = 0; k < kn; ++k) count16(col[k * PLANE + (((sh + k * pl) & 3) - sh)]);
         }
       }
       __syncthreads();
