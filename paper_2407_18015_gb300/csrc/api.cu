@@ -31,13 +31,15 @@ const char *kStatusText[] = {
 
 struct DeviceGuard {
   int prev = -1;
+  bool switched = false;
   cudaError_t err = cudaSuccess;
   explicit DeviceGuard(int dev) {
     if (cudaGetDevice(&prev) != cudaSuccess) prev = -1;
-    if (prev != dev) err = cudaSetDevice(dev);
+    switched = prev != dev;
+    if (switched) err = cudaSetDevice(dev);
   }
   ~DeviceGuard() {
-    if (prev >= 0) cudaSetDevice(prev);
+    if (switched && prev >= 0) cudaSetDevice(prev);
   }
 };
 

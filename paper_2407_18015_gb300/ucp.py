@@ -59,6 +59,8 @@ _I = ctypes.c_int
 def lib():
     """The loaded libucp.so (raises if it has not been built)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(LIB_PATH):
@@ -139,8 +141,12 @@ def _hptr(a, name="array"):
 
 
 def _stream(stream=None, device=None):
-    s = stream if stream is not None else torch.cuda.current_stream(device)
-    return s.cuda_stream
+    """Handle of `stream`, or of the current stream of `device` (None: the
+    current device) without building a torch.cuda.Stream for it."""
+    if stream is not None:
+        return stream.cuda_stream
+    idx = device.index if device is not None else None
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device() if idx is None else idx)
 
 
 def make_desc(model="uniform", bins=8, epan_width_scale=0.0, mc_samples=10000, seed=0x5EED,
@@ -263,8 +269,8 @@ def ucp_probability_models(ctx, ens, descs, cptypes, out_min, out_max, vertex_st
             (vertex_status is not None and len(vertex_status) != n):
         raise ValueError("one output per model")
     darr = (ucp_model_desc * n)(*descs)
-    arr = lambda ts, dt, nm: ctypes.cast((ctypes.c_void_p * n)(
-        *[_ptr(t, dt, name=nm) for t in ts]), ctypes.c_void_p)
+    parr = _P * n
+    arr = lambda ts, dt, nm: parr(*[_ptr(t, dt, name=nm) for t in ts])
     rc = lib().ucp_probability_models(
         ctx, _ptr(ens, torch.float32, name="ens"), ens.shape[0], H, W, darr, n, int(cptypes),
         arr(out_min, torch.float32, "out_min"), arr(out_max, torch.float32, "out_max"),
@@ -284,14 +290,13 @@ def ucp_probability_host_models(ctx, ens_host, descs, cptypes, out_min_host, out
             (status_host is not None and len(status_host) != n):
         raise ValueError("one output per model")
     darr = (ucp_model_desc * n)(*descs)
-    pmin = (ctypes.c_void_p * n)(*[_hptr(a, "out_min_host") for a in out_min_host])
-    pmax = (ctypes.c_void_p * n)(*[_hptr(a, "out_max_host") for a in out_max_host])
-    pst = None if status_host is None else \
-        (ctypes.c_void_p * n)(*[_hptr(a, "status_host") for a in status_host])
-    addr = lambda a: None if a is None else ctypes.cast(a, ctypes.c_void_p)
+    parr = _P * n
+    pmin = parr(*[_hptr(a, "out_min_host") for a in out_min_host])
+    pmax = parr(*[_hptr(a, "out_max_host") for a in out_max_host])
+    pst = None if status_host is None else parr(*[_hptr(a, "status_host") for a in status_host])
     rc = lib().ucp_probability_host_models(
-        ctx, _hptr(ens_host, "ens_host"), N, H, W, darr, n, int(cptypes), addr(pmin), addr(pmax),
-        addr(pst), _stream(stream))
+        ctx, _hptr(ens_host, "ens_host"), N, H, W, darr, n, int(cptypes), pmin, pmax, pst,
+        _stream(stream))
     _check(rc, "ucp_probability_host_models", ctx)
 
 
@@ -503,12 +508,14 @@ class UcpProbability(torch.autograd.Function):
         model, bins, boundary = ctx.desc_args
         desc = make_desc(model, bins=bins, boundary=boundary)
         c = default_context(params.device)
-        grad = c.backward(params.contiguous(), desc, ctx.cptype,
-                          grad_out.to(torch.float32).contiguous())
-        if desc.model == UCP_HISTOGRAM:
-            full = torch.zeros_like(params)
-            full[2:] = grad
-            grad = full
+        params, weight = params.contiguous(), grad_out.to(torch.float32).contiguous()
+        if desc.model != UCP_HISTOGRAM:
+            return c.backward(params, desc, ctx.cptype, weight), None, None, None, None
+        # the adjoint writes the masses' planes of the gradient in place; the
+        # support (lo, hi) is held fixed
+        grad = torch.empty_like(params)
+        grad[:2].zero_()
+        ucp_backward(c.handle, params, desc, ctx.cptype, weight, grad[2:])
         return grad, None, None, None, None
 
 
