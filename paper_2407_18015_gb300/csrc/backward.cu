@@ -1019,17 +1019,21 @@ __device__ __forceinline__ void hist_adj_walk(const float *sm, const float4 *R4,
     for (int i = 0; i < 4; ++i) e[i] = nw[i].nx();
     const float x1 = fmin5(e[0], e[1], e[2], e[3], dc.y);
     const float d = x1 - x0, hd = 0.5f * d, xm = x0 + hd;
-    const float2 hh = make_float2(hd, hd), nh = make_float2(-hd, -hd), nx2 = make_float2(-xm, -xm);
     // neighbours in the pairs (0, 2) and (1, 3): middle values m, half falls
-    // D, in-bin weights at the middle w and their half falls v
-    const float2 zA = make_float2(nw[0].r.z, nw[2].r.z), zB = make_float2(nw[1].r.z, nw[3].r.z);
-    const float2 gA = make_float2(nw[0].r.x, nw[2].r.x), gB = make_float2(nw[1].r.x, nw[3].r.x);
-    const float2 iA = make_float2(nw[0].r.y, nw[2].r.y), iB = make_float2(nw[1].r.y, nw[3].r.y);
-    const float2 mA = __ffma2_rn(zA, nh, gA), mB = __ffma2_rn(zB, nh, gB);
-    const float2 DA = __fmul2_rn(zA, hh), DB = __fmul2_rn(zB, hh);
-    const float2 vA = __fmul2_rn(iA, hh), vB = __fmul2_rn(iB, hh);
-    const float2 wA = __fmul2_rn(__fadd2_rn(make_float2(e[0], e[2]), nx2), iA);
-    const float2 wB = __fmul2_rn(__fadd2_rn(make_float2(e[1], e[3]), nx2), iB);
+    // D, in-bin weights at the middle w and their half falls v (scalar
+    // operations write the pairs' halves from the rows' registers; packed ones
+    // would first move their operands into pairs)
+    auto mid = [&](int i) { return fmaf(-nw[i].r.z, hd, nw[i].r.x); };
+    auto fall = [&](int i) { return nw[i].r.z * hd; };
+    auto wfall = [&](int i) { return nw[i].r.y * hd; };
+    const float2 nx2 = make_float2(-xm, -xm);
+    const float2 mA = make_float2(mid(0), mid(2)), mB = make_float2(mid(1), mid(3));
+    const float2 DA = make_float2(fall(0), fall(2)), DB = make_float2(fall(1), fall(3));
+    const float2 vA = make_float2(wfall(0), wfall(2)), vB = make_float2(wfall(1), wfall(3));
+    const float2 eA = __fadd2_rn(make_float2(e[0], e[2]), nx2);
+    const float2 eB = __fadd2_rn(make_float2(e[1], e[3]), nx2);
+    const float2 wA = make_float2(eA.x * nw[0].r.y, eA.y * nw[2].r.y);
+    const float2 wB = make_float2(eB.x * nw[1].r.y, eB.y * nw[3].r.y);
     // (01 | 23): products, cross terms / 3, U, V
     const float2 p = __fmul2_rn(mA, mB), g = __fmul2_rn(DA, DB);
     const float2 b = __ffma2_rn(mA, DB, __fmul2_rn(mB, DA)), b3 = __fmul2_rn(b, third);
