@@ -907,7 +907,7 @@ __global__ void __launch_bounds__(NTHREADS, 2)
 // shared memory).  One running partial per neighbour, A = C(start of its bin)
 // + in-bin integral, scaled by the centre's weight, is stored as it is and
 // restarted at C; the rows carry 1/h, whose 0 also says that the walker is
-// not inside a bin.  2048 x 2048 vertices, 16 bins: 2.83 -> 2.31 ms (three
+// not inside a bin.  2048 x 2048 vertices, 16 bins: 2.83 -> 2.26 ms (three
 // Gauss-Legendre nodes, the partial in two parts and a width per walker
 // before).
 

@@ -113,17 +113,25 @@ __global__ void __launch_bounds__(256) fit_kernel(Field f) {
   }
 }
 
-// Histogram fit of at most 16 bins and MAXN members in one pass over the
-// members: a thread holds its vertex's members in registers (every load in
+// Histogram fit of at most RB bins (8 or 16) and MAXN members in one pass over
+// the members: a thread holds its vertex's members in registers (every load in
 // flight at once), takes their minimum and maximum (NaN-propagating: a
 // non-finite member shows in them) and bins them from the registers, where
-// fit_kernel reads them twice.  The same values as fit_kernel: the same
-// bins, counters and count / N table.
-template <int MAXN>
+// fit_kernel reads them twice.  The same values as fit_kernel: the same bins,
+// 8-bit counters and count / N table.  Up to 8 bins count in one 64-bit word;
+// 16 add one of sixteen 16-byte increments read from shared memory (a read and
+// four additions, instead of shifts and selects between two words).
+template <int MAXN, int RB>
 __global__ void __launch_bounds__(128) fit_hist_regs(Field f) {
   __shared__ float mtab[MAXN + 1];
+  __shared__ uint4 itab[16];
   const int N = f.N, B = f.B;
   for (int c = threadIdx.x; c <= N; c += blockDim.x) mtab[c] = __fdiv_rn((float)c, (float)N);
+  if (RB > 8 && threadIdx.x < 16) {
+    const unsigned j = threadIdx.x, one = 1u << (8 * (j & 3));
+    itab[j] = make_uint4(j < 4 ? one : 0u, j / 4 == 1 ? one : 0u, j / 4 == 2 ? one : 0u,
+                         j / 4 == 3 ? one : 0u);
+  }
   __syncthreads();
   const long long plane = f.plane;
   float *out = const_cast<float *>(f.params);
@@ -150,27 +158,40 @@ __global__ void __launch_bounds__(128) fit_hist_regs(Field f) {
       for (int q = 0; q < 2 + B; ++q) out[q * plane + i] = __int_as_float(0x7fc00000);
       st |= V_NONFINITE;
     } else {
-      unsigned long long c0 = 0ull, c1 = 0ull;
+      uint4 c = make_uint4(0u, 0u, 0u, 0u);
       if (mn == mx) {
-        c0 = (unsigned long long)N;
+        c.x = (unsigned)N;
         st |= V_DEGENERATE;
       } else {
         const float sc = __fdiv_rn((float)B, __fsub_rn(mx, mn));
+        unsigned long long c8 = 0ull;
 #pragma unroll
         for (int k = 0; k < MAXN; ++k) {
           if (k < N) {
             const int j = hist_bin_nonneg(v[k], mn, sc, B);
-            const unsigned long long inc = 1ull << ((j & 7) << 3);
-            c0 += j < 8 ? inc : 0ull;
-            c1 += j < 8 ? 0ull : inc;
+            if constexpr (RB == 8) {
+              c8 += 1ull << (j << 3);
+            } else {
+              const uint4 inc = itab[j];
+              c.x += inc.x;
+              c.y += inc.y;
+              c.z += inc.z;
+              c.w += inc.w;
+            }
           }
+        }
+        if constexpr (RB == 8) {
+          c.x = (unsigned)c8;
+          c.y = (unsigned)(c8 >> 32);
         }
       }
       out[i] = mn;
       out[plane + i] = mx;
-      for (int q = 0; q < B; ++q) {
-        const unsigned c = (unsigned)((q < 8 ? c0 : c1) >> ((q & 7) << 3)) & 255u;
-        out[(2 + q) * plane + i] = mtab[c];
+      float *o = out + 2 * plane + i;
+#pragma unroll
+      for (int q = 0; q < RB; ++q) {
+        const unsigned w = q < 4 ? c.x : (q < 8 ? c.y : (q < 12 ? c.z : c.w));
+        if (q < B) o[q * plane] = mtab[(w >> ((q & 3) << 3)) & 255u];
       }
     }
     if (f.status) f.status[i] = st;
@@ -276,8 +297,13 @@ cudaError_t launch_fit(const Field &f, int model, cudaStream_t s) {
     case kSemi:
       if (f.B <= 16 && f.N >= 1 && f.N <= 64) {
         const int g2 = grid_for(f.plane, 128);
-        if (f.N <= 32) fit_hist_regs<32><<<g2, 128, 0, s>>>(f);
-        else fit_hist_regs<64><<<g2, 128, 0, s>>>(f);
+        if (f.B <= 8) {
+          if (f.N <= 32) fit_hist_regs<32, 8><<<g2, 128, 0, s>>>(f);
+          else fit_hist_regs<64, 8><<<g2, 128, 0, s>>>(f);
+        } else {
+          if (f.N <= 32) fit_hist_regs<32, 16><<<g2, 128, 0, s>>>(f);
+          else fit_hist_regs<64, 16><<<g2, 128, 0, s>>>(f);
+        }
       } else {
         fit_kernel<kHist><<<g, 256, 0, s>>>(f);
       }
