@@ -1128,19 +1128,23 @@ __device__ __forceinline__ void semi_tails(const float *sm, const SemiNb &n, int
   }
 }
 
-// The same for a neighbour with bins, or an absent one that is described as
-// one with F = 1 at every x (ih = 0, T = 2, its P_0 a cell that holds 1):
-// the position in bins is clamped to [0, B], where P_0 = 0 and P_B = T are
-// the tails outside the support, and its whole part comes from the mantissa
-// of v + 2^23 rounded down (no conversion instructions, which run at a
-// quarter of the rate).  Two shared reads at one address.
+// F_n(x) for a neighbour with bins, or an absent one that is described as one
+// with F = 1 at every x (iw = 0, T = 2, its P_0 a cell that holds 1): the
+// position in the support is clamped to [0, 1] (the multiply's saturation),
+// where P_0 = 0 and P_B = T are the tails outside the support; its whole part
+// in bins comes from the mantissa of v B + 2^23 rounded down (no conversion
+// instructions, which run at a quarter of the rate).  Two shared reads at one
+// address; base: the shared-memory address of P_0, less that of 2^23 bins.
 constexpr uint32_t kTwo23 = 0x4B000000u;  // 2^23 as binary32
 template <int WS>
-__device__ __forceinline__ float semi_cdf(const float *sm, const SemiNb &n, float Bf, float x) {
-  const float v = fminf(fmaxf((x - n.lam) * n.ih, 0.f), Bf);
-  const float t = __fadd_rz(v, 8388608.f);
-  const float *row = sm + (n.off + (int)((__float_as_uint(t) - kTwo23) * (2 * WS)));
-  return fmaf(row[WS], v - (t - 8388608.f), row[0]);
+__device__ __forceinline__ float semi_cdf(uint32_t base, float lam, float iw, float Bf, float x) {
+  const float v = __saturatef((x - lam) * iw);
+  const float t = __fmaf_rz(v, Bf, 8388608.f);
+  const uint32_t a = __float_as_uint(t) * (8u * WS) + base;
+  float P, m;
+  asm("ld.shared.f32 %0, [%1];" : "=f"(P) : "r"(a));
+  asm("ld.shared.f32 %0, [%1 + %2];" : "=f"(m) : "r"(a), "n"(4 * WS));
+  return fmaf(m, fmaf(v, Bf, 8388608.f - t), P);
 }
 
 // The bin of a sample: the number of running sums P_1..P_B that are <= t,
@@ -1162,47 +1166,49 @@ __device__ __forceinline__ int semi_bin(const float *P0, int B, float t) {
   }
 }
 
-// Sums over the samples (min, max; saddle: in the first alone).  PM: a
+// Sums over the samples (min, max; saddle: in the first alone; both halves of
+// the packed FP32 arithmetic).  PM: a
 // present neighbour is a point mass (rare: the general tails).
 // Bound by instruction issue; per sample half a Philox block (ten 64-bit
 // products, four FP32-pipe cycles each), log2 B probes and four tails of two
-// reads: 1024 x 1024 x 20, 8 bins, 1000 samples 4.03 ms (7.57
+// reads: 1024 x 1024 x 20, 8 bins, 1000 samples 3.87 ms (7.57
 // with the general tails and a data-dependent search loop).
 template <int WS, bool SADDLE, int LOG, bool PM>
 __device__ __forceinline__ void semi_sums(const float *sm, int l, float h1, const SemiNb *nb,
                                           int B, int S, float T1, const PhiloxKeys &K,
-                                          uint32_t vid, uint32_t field, const int *sg, Kahan &amin,
-                                          Kahan &amax) {
+                                          uint32_t vid, uint32_t field, const int *sg,
+                                          float2 &sums) {
   const float Bf = (float)B;
   const float *P0 = sm + 2 * WS + l;
+  uint32_t base[4];
+  float iw[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    base[i] = static_cast<uint32_t>(__cvta_generic_to_shared(sm + nb[i].off)) - kTwo23 * (8u * WS);
+    iw[i] = nb[i].ih * (1.f / Bf);
+  }
+  Kahan2 acc;
   auto sample = [&](uint32_t wa, uint32_t wb) {
     const int j = semi_bin<WS, LOG>(P0, B, u01(wa) * T1);
     const float jf = __uint_as_float(kTwo23 + (uint32_t)j) - 8388608.f;
     const float x = (jf + u01(wb)) * h1;
-    float pm = T1, pM = T1;
+    float2 p = make_float2(T1, T1);  // (minimum, maximum) or the saddle's terms
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       float G, F;
       if constexpr (PM) {
         semi_tails<WS>(sm, nb[i], B, x, G, F);
       } else {
-        F = semi_cdf<WS>(sm, nb[i], Bf, x);
+        F = semi_cdf<WS>(base[i], nb[i].lam, iw[i], Bf, x);
         G = nb[i].T - F;
       }
-      if constexpr (SADDLE) {
-        pm *= sg[i] > 0 ? G : (sg[i] < 0 ? F : 1.f);
-        pM *= sg[i] > 0 ? F : (sg[i] < 0 ? G : 1.f);
-      } else {
-        pm *= G;
-        pM *= F;
-      }
+      float2 f = make_float2(G, F);
+      if constexpr (SADDLE)
+        f = sg[i] > 0 ? f : (sg[i] < 0 ? make_float2(F, G) : make_float2(1.f, 1.f));
+      p = __fmul2_rn(p, f);
     }
-    if constexpr (SADDLE) {
-      amin.add(pm + pM);
-    } else {
-      amin.add(pm);
-      amax.add(pM);
-    }
+    if constexpr (SADDLE) p.x += p.y;
+    acc.add(p);
   };
   const int pairs = S >> 1;
   for (int s = 0; s < pairs; ++s) {
@@ -1214,6 +1220,7 @@ __device__ __forceinline__ void semi_sums(const float *sm, int l, float h1, cons
     const uint4 r = philox_block(make_uint4((uint32_t)pairs, vid, field, 2u), K);
     sample(r.x, r.y);
   }
+  sums = acc.s;
 }
 
 // sm: the tile's rows (see semi_rows); l: the centre
@@ -1242,19 +1249,19 @@ __device__ __forceinline__ void semi_vertex(const float *sm, int l, float lo1, f
     return;
   }
   const float h1 = (hi1 - lo1) / (float)B;
-  Kahan amin, amax;
+  float2 sums;
   const bool pm = nb[0].kind == 2 || nb[1].kind == 2 || nb[2].kind == 2 || nb[3].kind == 2;
   if (pm)
-    semi_sums<WS, SADDLE, 0, true>(sm, l, h1, nb, B, S, T1, K, vid, field, sg, amin, amax);
+    semi_sums<WS, SADDLE, 0, true>(sm, l, h1, nb, B, S, T1, K, vid, field, sg, sums);
   else if (B == 8)
-    semi_sums<WS, SADDLE, 3, false>(sm, l, h1, nb, B, S, T1, K, vid, field, sg, amin, amax);
+    semi_sums<WS, SADDLE, 3, false>(sm, l, h1, nb, B, S, T1, K, vid, field, sg, sums);
   else if (B == 16)
-    semi_sums<WS, SADDLE, 4, false>(sm, l, h1, nb, B, S, T1, K, vid, field, sg, amin, amax);
+    semi_sums<WS, SADDLE, 4, false>(sm, l, h1, nb, B, S, T1, K, vid, field, sg, sums);
   else
-    semi_sums<WS, SADDLE, 0, false>(sm, l, h1, nb, B, S, T1, K, vid, field, sg, amin, amax);
+    semi_sums<WS, SADDLE, 0, false>(sm, l, h1, nb, B, S, T1, K, vid, field, sg, sums);
   const float inv = 1.f / (float)S;
-  pmin = amin.get() * inv;
-  pmax = amax.get() * inv;
+  pmin = sums.x * inv;
+  pmax = sums.y * inv;
   psad = pmin;
 }
 
