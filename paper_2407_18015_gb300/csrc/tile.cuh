@@ -28,11 +28,11 @@ __host__ __device__ constexpr long long tile_floats(int model, int B, int TYv) {
 // written once the rows are built); while the rows are built from masses
 // held in the tile (rows 2 .. 1 + B), those take their place, else (masses
 // from bin counts in registers) a table of the values count / N follows,
-// then, for more than 8 bins, the counters' increments per bin
-// (ROWS_INC_TABLE floats: 16 bins x two 64-bit words).  The rows themselves
+// then, for more than 8 bins, the counters' increments (ROWS_INC_TABLE floats:
+// eight 64-bit words).  The rows themselves
 // (hist_r4_rows x hist_r4_stride float4) come on top.
 constexpr int ROWS_MASS_TABLE = 256;
-constexpr int ROWS_INC_TABLE = 64;
+constexpr int ROWS_INC_TABLE = 16;
 __host__ __device__ constexpr long long hist_rows_tile_floats(int B, int TYv, bool masses) {
   const long long halo = (long long)(TYv + 2) * 34;
   return masses ? (2 + B > 4 ? 2 + B : 4) * halo
@@ -747,19 +747,20 @@ __device__ __forceinline__ bool stage_members_tma(const Field &f, float *sm, flo
   }
   if constexpr (MODEL == kHist && RB > 0) {
     // the masses count / N of up to 255 members (see the per-bin rows
-    // below), and for more than 8 bins each bin's increment of the two
-    // words of 8-bit counters: bin j adds 1 << 8 (j mod 8) to word j / 8
-    // (one 16-byte read instead of a shift and two selects per member;
-    // with one word the shift is cheaper: 162.5 vs 169 us at 1024 x 1024 x
-    // 20, 8 bins, against 1397 -> 1367 us at 2048 x 2048 x 50, 16 bins)
+    // below), and for more than 8 bins the eight increments 1 << 8 (j mod 8)
+    // of a 64-bit word of counters, read from shared memory (64 bytes: no two
+    // entries share a bank) and added to the word of bin j under a predicate
+    // (with one word the shift is cheaper; a table of sixteen 16-byte
+    // increments for both words took 71 us of bank conflicts at 1021 x 1023 x
+    // 50, 16 bins; the 64-field batch with 16 bins 3.15 -> 3.03 ms)
     if (N <= 255) {
       for (int c = threadIdx.x; c <= N; c += NTHREADS)
         sm[4 * HALO + c] = __fdiv_rn((float)c, (float)N);
       if constexpr (RB > 8) {
-        ulonglong2 *itab = reinterpret_cast<ulonglong2 *>(sm + 4 * HALO + ROWS_MASS_TABLE);
-        for (int j = threadIdx.x; j < RB; j += NTHREADS)
-          itab[j] = make_ulonglong2(j < 8 ? 1ull << (j << 3) : 0ull,
-                                    j < 8 ? 0ull : 1ull << ((j - 8) << 3));
+        if (threadIdx.x < 8)
+          reinterpret_cast<uint2 *>(sm + 4 * HALO + ROWS_MASS_TABLE)[threadIdx.x] =
+              make_uint2(threadIdx.x < 4 ? 1u << (8 * threadIdx.x) : 0u,
+                         threadIdx.x < 4 ? 0u : 1u << (8 * threadIdx.x - 32));
       }
     }
   }
@@ -893,8 +894,10 @@ __device__ __forceinline__ bool stage_members_tma(const Field &f, float *sm, flo
     bool bin[PER];
     bool any = false;
     unsigned long long cw[PER][NW16];
+    uint4 c32[PER];  // more than 8 bins: the two words of 8-bit counters
 #pragma unroll
     for (int p = 0; p < PER; ++p) {
+      c32[p] = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
       for (int w = 0; w < NW16; ++w) cw[p][w] = 0ull;
       bin[p] = in[p] && !nf[p] && mn[p] != mx[p];
@@ -917,16 +920,21 @@ __device__ __forceinline__ bool stage_members_tma(const Field &f, float *sm, flo
           if (!bin[p]) continue;
           const int sh = shift0(p, k0);
           const float *col = box + off[p] + sh;
-          const ulonglong2 *itab =
-              reinterpret_cast<const ulonglong2 *>(sm + 4 * HALO + ROWS_MASS_TABLE);
+          const uint2 *itab = reinterpret_cast<const uint2 *>(sm + 4 * HALO + ROWS_MASS_TABLE);
           auto count8 = [&](float v) {
             const int j = hist_bin_nonneg(v, mn[p], sc[p], B);
             if constexpr (NW8 == 1) {
               cw[p][0] += 1ull << ((j & 7) << 3);
             } else {
-              const ulonglong2 inc = itab[j];
-              cw[p][0] += inc.x;
-              cw[p][1] += inc.y;
+              // byte counters never carry: the words' halves add apart
+              const uint2 inc = itab[j & 7];
+              if (j < 8) {
+                c32[p].x += inc.x;
+                c32[p].y += inc.y;
+              } else {
+                c32[p].z += inc.x;
+                c32[p].w += inc.y;
+              }
             }
           };
           auto count16 = [&](float v) {
@@ -953,7 +961,12 @@ __device__ __forceinline__ bool stage_members_tma(const Field &f, float *sm, flo
       if (!in[p]) continue;
       hist_row_table_counts<HALO, RS, RB>(
           sm, R4, lv[p], B, nf[p], mn[p], mx[p], [&](int k) -> float {
-            if (!wide) return mtab[(unsigned)(cw[p][k >> 3] >> ((k & 7) << 3)) & 255u];
+            if (!wide) {
+              if constexpr (NW8 == 1)
+                return mtab[(unsigned)(cw[p][0] >> ((k & 7) << 3)) & 255u];
+              const unsigned w = k < 4 ? c32[p].x : (k < 8 ? c32[p].y : (k < 12 ? c32[p].z : c32[p].w));
+              return mtab[(w >> ((k & 3) << 3)) & 255u];
+            }
             return __fdiv_rn((float)((unsigned)(cw[p][k >> 2] >> ((k & 3) << 4)) & 0xFFFFu),
                              (float)N);
           });
