@@ -227,6 +227,8 @@ __global__ void __launch_bounds__(NTHREADS, (TileOcc<MODEL, RB>::value))
   if constexpr (ROWS)
     R4 = reinterpret_cast<float4 *>(
         sm + ((param_tile_floats<MODEL, TYm, ROWS>(f.B, FROM_MEMBERS) + 3) & ~3LL));
+  if constexpr (MODEL == kSemi)
+    R4 = reinterpret_cast<float4 *>(sm + ((tile_floats(MODEL, f.B, TYm) + 3) & ~3LL));
   process_tile<MODEL, FROM_MEMBERS, TYm, SADDLE, false, RB>(
       f, f.y0 + (tile / tiles_x) * TYm, (tile % tiles_x) * TX, sm, nullptr, nullptr, nullptr, R4);
 }
@@ -255,13 +257,13 @@ __global__ void __launch_bounds__(NTHREADS, (TmaOcc<MODEL, SADDLE, RB>::value))
   const int tile = blockIdx.x;
   const int box_floats = f.tma_nc * (TYm + 2) * kBoxW;
   constexpr bool ROWS = RB > 0;
-  const int r4 = ROWS ? r4_floats(f.B, TYm) : 0;
+  const int r4 = ROWS ? r4_floats(f.B, TYm) : (MODEL == kSemi ? semi_tab_floats(f.B, TYm) : 0);
   float *sm = smem + max(box_floats, r4);
   const long long tile_f = param_tile_floats<MODEL, TYm, ROWS>(f.B, false);
   uint64_t *bar = reinterpret_cast<uint64_t *>(sm + ((tile_f + 1) & ~1LL));
   process_tile<MODEL, true, TYm, SADDLE, true, RB, ASYNC>(
       f, f.y0 + (tile / tiles_x) * TYm, (tile % tiles_x) * TX, sm, &tmap, smem, bar,
-      ROWS ? reinterpret_cast<float4 *>(smem) : nullptr);
+      ROWS || MODEL == kSemi ? reinterpret_cast<float4 *>(smem) : nullptr);
 }
 
 // ---------------------------------------------------------------------------
@@ -332,6 +334,15 @@ static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 
 void *tensor_map_encoder_fn() { return reinterpret_cast<void *>(tensor_map_encoder()); }
 
+// Shared-memory bytes a CTA may take at the model's occupancy; the estimator's
+// table and parameter tile of more than 12 bins leave room for three CTAs per
+// SM only (16 bins: 72 KB).
+template <int MODEL, int RB>
+static size_t tile_budget(int B) {
+  const int occ = MODEL == kSemi && semi_apart(B) && B > 12 ? 3 : TileOcc<MODEL, RB>::value;
+  return (size_t)227 * 1024 / occ - 1024;
+}
+
 // Members per TMA box next to a TYm-row parameter tile at the model's
 // occupancy (0: not even one), capped at N and at the box limit of 256.
 template <int MODEL, int TYm, int RB>
@@ -340,7 +351,7 @@ static int tma_box_members(int N, int B) {
   const size_t tile_b =
       (size_t)((param_tile_floats<MODEL, TYm, ROWS>(B, false) + 1) & ~1LL) * sizeof(float) + 16;
   const size_t per_member = (size_t)(TYm + 2) * kBoxW * sizeof(float);
-  const size_t budget = (size_t)227 * 1024 / TileOcc<MODEL, RB>::value - 1024;
+  const size_t budget = tile_budget<MODEL, RB>(B);
   if (budget < tile_b + per_member) return 0;
   const size_t nc = (budget - tile_b) / per_member;
   return (int)std::min<size_t>(nc, (size_t)std::min(N, 256));
@@ -362,10 +373,11 @@ static bool launch_tile_tma(const Field &f, int tiles_x, int tiles, cudaStream_t
   const size_t tile_b =
       (size_t)((param_tile_floats<MODEL, TYm, ROWS>(f.B, false) + 1) & ~1LL) * sizeof(float) + 16;
   const size_t per_member = (size_t)(TYm + 2) * kBoxW * sizeof(float);
-  const size_t budget = (size_t)227 * 1024 / TileOcc<MODEL, RB>::value - 1024;
+  const size_t budget = tile_budget<MODEL, RB>(f.B);
   const int nc = tma_box_members<MODEL, TYm, RB>(f.N, f.B);
   if (nc < 1) return false;
-  const size_t r4_b = ROWS ? (size_t)r4_floats(f.B, TYm) * sizeof(float) : 0;
+  const size_t r4_b = ROWS ? (size_t)r4_floats(f.B, TYm) * sizeof(float)
+                           : (MODEL == kSemi ? (size_t)semi_tab_floats(f.B, TYm) * sizeof(float) : 0);
   if (tile_b + r4_b > budget) return false;
   CUtensorMap map;
   memset(&map, 0, sizeof(map));
@@ -462,6 +474,9 @@ static cudaError_t launch_tile_h(const Field &f, cudaStream_t s) {
   if constexpr (RB > 0)
     smem = (size_t)((param_tile_floats<MODEL, TYm, true>(f.B, FM) + 3) & ~3LL) * sizeof(float) +
            (size_t)r4_floats(f.B, TYm) * sizeof(float);
+  if constexpr (MODEL == kSemi)
+    smem = (size_t)((tile_floats(MODEL, f.B, TYm) + 3) & ~3LL) * sizeof(float) +
+           (size_t)semi_tab_floats(f.B, TYm) * sizeof(float);
   // per device: the attribute is set once (several host threads may race to
   // set it; setting it twice is harmless, the flag itself is atomic)
   static std::atomic<bool> attr_set[128] = {};
@@ -474,7 +489,7 @@ static cudaError_t launch_tile_h(const Field &f, cudaStream_t s) {
     // table, total, status and ordering scratch, the estimator its running
     // mass sums: 95 KB and 173 KB at 10 x 34), or the per-bin rows' bound
     const size_t most = std::max((size_t)tile_floats(MODEL, kMaxBins, TYm) * sizeof(float),
-                                 MODEL == kHist ? (size_t)227 * 1024 : (size_t)0);
+                                 hist_params(MODEL) ? (size_t)227 * 1024 : (size_t)0);
     e = cudaFuncSetAttribute(tile_kernel<MODEL, FM, SADDLE, TYm, RB>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
     if (e != cudaSuccess) {

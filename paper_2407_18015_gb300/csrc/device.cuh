@@ -1098,27 +1098,34 @@ __device__ __forceinline__ float u01(uint32_t r) {
 // (binary32, bin order) that are <= ua * T_1, clamped to B - 1 (binary
 // search); position: (j + ub) h inside the bin.
 
-// Rows of a staged vertex (row r at sm[r * WS + l]): 0 lo, 1 hi, 2 + 2k the
-// running mass sum P_k = m_0 + ... + m_{k-1} (k = 0..B, in bin order), 3 + 2k
-// the mass m_k (m_B = 0).  An absent neighbour reads P_0 and m_0 of the halo's
-// first corner (no vertex's neighbour), which hold 1 and 0.
-__host__ __device__ constexpr int semi_rows(int B) { return 4 + 2 * B; }
+// Table of a staged vertex l, rows WS floats apart (row r at tab[r * WS + l]):
+// 2k the running mass sum P_k = m_0 + ... + m_{k-1} (k = 0..B, in bin order),
+// 2k + 1 the mass m_k (m_B = 0).  An absent neighbour reads P_0 and m_0 of the
+// halo's first corner (no vertex's neighbour), which hold 1 and 0.
+// Up to 16 bins the table is apart from the parameter tile with rows a
+// multiple of 32 floats apart, so that the bank of a read depends on the
+// vertex alone: the lanes of a warp, consecutive vertices on any rows, never
+// share one.  More bins (whose two copies of the masses would not fit) keep
+// it in the parameter tile's own rows, in the masses' place.
+__host__ __device__ constexpr int semi_rows(int B) { return 2 + 2 * B; }
+__host__ __device__ constexpr bool semi_apart(int B) { return B <= 16; }
+__host__ __device__ constexpr int semi_stride(int halo) { return (halo + 31) & ~31; }
 
 struct SemiNb {
   float lam, ih, T;  // local support start, B / (hi - lo), total mass
-  int off;           // shared-memory index of its P_0
+  int off;           // its column in the table
   int kind;          // 0 absent, 1 bins, 2 point mass
 };
 
 // F_n(x) and G_n(x) = T_n - F_n(x) of a neighbour of any kind at the local
 // position x.
 template <int WS>
-__device__ __forceinline__ void semi_tails(const float *sm, const SemiNb &n, int B, float x,
+__device__ __forceinline__ void semi_tails(const float *tab, const SemiNb &n, int B, float x,
                                            float &G, float &F) {
   const float v = (x - n.lam) * n.ih;
   const float fk = floorf(v);
   const int k = (int)fminf(fmaxf(fk, 0.f), (float)(B - 1));
-  const float *row = sm + n.off + (n.kind == 1 ? 2 * k * WS : 0);
+  const float *row = tab + n.off + (n.kind == 1 ? 2 * k * WS : 0);
   const float Fin = fmaf(row[WS], v - fk, row[0]);
   F = fk < 0.f ? 0.f : (fk >= (float)B ? n.T : Fin);
   G = fk < 0.f ? n.T : (fk >= (float)B ? 0.f : n.T - Fin);
@@ -1150,7 +1157,7 @@ __device__ __forceinline__ float semi_cdf(uint32_t base, float lam, float iw, fl
 // The bin of a sample: the number of running sums P_1..P_B that are <= t,
 // clamped to B - 1.  The sums never fall, so this is a binary search over
 // P_1..P_{B-1}; with B = 2^LOG every probe is one of them and costs a read at
-// a constant offset, a compare and a predicated add.
+// a constant offset, a compare and a predicated add.  LOG < 0: any B <= 2^-LOG.
 template <int WS, int LOG>
 __device__ __forceinline__ int semi_bin(const float *P0, int B, float t) {
   int pos = 0;
@@ -1160,7 +1167,8 @@ __device__ __forceinline__ int semi_bin(const float *P0, int B, float t) {
       if (P0[(pos + st) * (2 * WS)] <= t) pos += st;
     return pos;
   } else {
-    for (int st = 32; st > 0; st >>= 1)
+#pragma unroll
+    for (int st = 1 << (-LOG - 1); st > 0; st >>= 1)
       if (pos + st < B && P0[(pos + st) * (2 * WS)] <= t) pos += st;
     return pos;
   }
@@ -1171,20 +1179,20 @@ __device__ __forceinline__ int semi_bin(const float *P0, int B, float t) {
 // present neighbour is a point mass (rare: the general tails).
 // Bound by instruction issue; per sample half a Philox block (ten 64-bit
 // products, four FP32-pipe cycles each), log2 B probes and four tails of two
-// reads: 1024 x 1024 x 20, 8 bins, 1000 samples 3.87 ms (7.57
+// reads: 1024 x 1024 x 20, 8 bins, 1000 samples 3.40 ms (7.57
 // with the general tails and a data-dependent search loop).
 template <int WS, bool SADDLE, int LOG, bool PM>
-__device__ __forceinline__ void semi_sums(const float *sm, int l, float h1, const SemiNb *nb,
+__device__ __forceinline__ void semi_sums(const float *tab, int l, float h1, const SemiNb *nb,
                                           int B, int S, float T1, const PhiloxKeys &K,
                                           uint32_t vid, uint32_t field, const int *sg,
                                           float2 &sums) {
   const float Bf = (float)B;
-  const float *P0 = sm + 2 * WS + l;
+  const float *P0 = tab + l;
   uint32_t base[4];
   float iw[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    base[i] = static_cast<uint32_t>(__cvta_generic_to_shared(sm + nb[i].off)) - kTwo23 * (8u * WS);
+    base[i] = static_cast<uint32_t>(__cvta_generic_to_shared(tab + nb[i].off)) - kTwo23 * (8u * WS);
     iw[i] = nb[i].ih * (1.f / Bf);
   }
   Kahan2 acc;
@@ -1197,7 +1205,7 @@ __device__ __forceinline__ void semi_sums(const float *sm, int l, float h1, cons
     for (int i = 0; i < 4; ++i) {
       float G, F;
       if constexpr (PM) {
-        semi_tails<WS>(sm, nb[i], B, x, G, F);
+        semi_tails<WS>(tab, nb[i], B, x, G, F);
       } else {
         F = semi_cdf<WS>(base[i], nb[i].lam, iw[i], Bf, x);
         G = nb[i].T - F;
@@ -1223,19 +1231,19 @@ __device__ __forceinline__ void semi_sums(const float *sm, int l, float h1, cons
   sums = acc.s;
 }
 
-// sm: the tile's rows (see semi_rows); l: the centre
-template <int WS, bool SADDLE>
-__device__ __forceinline__ void semi_vertex(const float *sm, int l, float lo1, float hi1,
+// tab: the tile's table; l: the centre
+template <int WS, bool SADDLE, bool APART>
+__device__ __forceinline__ void semi_vertex(const float *tab, int l, float lo1, float hi1,
                                             const SemiNb *nb, int B, int S, const PhiloxKeys &K,
                                             uint32_t vid, uint32_t field, const int *sg,
                                             float &pmin, float &pmax, float &psad) {
-  const float T1 = sm[(2 + 2 * B) * WS + l];
+  const float T1 = tab[2 * B * WS + l];
   if (lo1 == hi1) {  // point-mass centre: every sample is its position
     float gm = T1, gM = T1, t1 = T1, t2 = T1;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       float G, F;
-      semi_tails<WS>(sm, nb[i], B, 0.f, G, F);
+      semi_tails<WS>(tab, nb[i], B, 0.f, G, F);
       gm *= G;
       gM *= F;
       if (SADDLE && sg[i] != 0) {
@@ -1252,13 +1260,13 @@ __device__ __forceinline__ void semi_vertex(const float *sm, int l, float lo1, f
   float2 sums;
   const bool pm = nb[0].kind == 2 || nb[1].kind == 2 || nb[2].kind == 2 || nb[3].kind == 2;
   if (pm)
-    semi_sums<WS, SADDLE, 0, true>(sm, l, h1, nb, B, S, T1, K, vid, field, sg, sums);
-  else if (B == 8)
-    semi_sums<WS, SADDLE, 3, false>(sm, l, h1, nb, B, S, T1, K, vid, field, sg, sums);
-  else if (B == 16)
-    semi_sums<WS, SADDLE, 4, false>(sm, l, h1, nb, B, S, T1, K, vid, field, sg, sums);
+    semi_sums<WS, SADDLE, -6, true>(tab, l, h1, nb, B, S, T1, K, vid, field, sg, sums);
+  else if (APART && B == 8)
+    semi_sums<WS, SADDLE, 3, false>(tab, l, h1, nb, B, S, T1, K, vid, field, sg, sums);
+  else if (APART && B == 16)
+    semi_sums<WS, SADDLE, 4, false>(tab, l, h1, nb, B, S, T1, K, vid, field, sg, sums);
   else
-    semi_sums<WS, SADDLE, 0, false>(sm, l, h1, nb, B, S, T1, K, vid, field, sg, sums);
+    semi_sums<WS, SADDLE, APART ? -4 : -6, false>(tab, l, h1, nb, B, S, T1, K, vid, field, sg, sums);
   const float inv = 1.f / (float)S;
   pmin = sums.x * inv;
   pmax = sums.y * inv;

@@ -18,7 +18,7 @@ __device__ __forceinline__ float qnan() { return __int_as_float(0x7fc00000); }
 // scratch of the walk ordering (buckets, then two 16-bit arrays of TYv x 32)
 __host__ __device__ constexpr long long tile_floats(int model, int B, int TYv) {
   const long long halo = (long long)(TYv + 2) * 34;
-  return model == kSemi   ? semi_rows(B) * halo
+  return model == kSemi   ? (2 + (semi_apart(B) ? B : semi_rows(B))) * halo
          : model == kHist ? hist_rows(B) * halo + kSortBuckets + TYv * 32
                           : 2 * halo;
 }
@@ -57,6 +57,11 @@ struct TileOcc {
 template <int MODEL, int TYm, bool ROWS>
 __host__ __device__ constexpr long long param_tile_floats(int B, bool masses) {
   return ROWS ? hist_rows_tile_floats(B, TYm, masses) : tile_floats(MODEL, B, TYm);
+}
+
+// floats of the estimator's table apart from the parameter tile (0: in it)
+__host__ __device__ constexpr int semi_tab_floats(int B, int TYv) {
+  return semi_apart(B) ? semi_rows(B) * semi_stride((TYv + 2) * 34) : 0;
 }
 
 // rows of a histogram tile's per-bin tables (hist_r4_rows float4 per halo
@@ -1054,7 +1059,7 @@ __device__ __forceinline__ uint8_t check_params(const float *sm, int l, int B, f
   uint8_t st = a > b ? V_BAD : (a == b ? V_DEGENERATE : 0);
   float t = 0.f;
   for (int q = 0; q < B; ++q) {
-    const float w = sm[(3 + 2 * q) * HALO + l];  // the estimator's rows
+    const float w = sm[(semi_apart(B) ? 2 + q : 3 + 2 * q) * HALO + l];  // the estimator's
     if (!isfinite(w)) st |= V_NONFINITE;
     else if (w < 0.f) st |= V_BAD;
     t += w;
@@ -1099,7 +1104,8 @@ __device__ __forceinline__ void integrate_tile(const Field &f, int ty0, int tx0,
 // of at most RB bins): the walk runs over per-bin rows in R4 (hist_r4_rows
 // rows of hist_r4_stride float4, 16-byte aligned; it may overlap `box`)
 // instead of the segment walker's tail table; each kernel instance carries
-// one of the two walks.
+// one of the two walks.  The estimator keeps its table there too
+// (semi_tab_floats).
 template <int MODEL, bool FROM_MEMBERS, int TYv, bool SADDLE = false, bool TMA = false,
           int RB = 0, bool ASYNC = false>
 __device__ __forceinline__ bool process_tile(const Field &f, int ty0, int tx0, float *sm,
@@ -1176,24 +1182,44 @@ __device__ __forceinline__ void integrate_tile(const Field &f, int ty0, int tx0,
     __syncthreads();
   }
   if constexpr (MODEL == kSemi) {
-    // the rows of semi_rows from the masses staged in rows 2 .. 1 + B: masses
-    // moved up to every other row (from the last: a mass moves to a row
-    // above those not yet moved), then the running sums in bin order
-    for (int l = threadIdx.x; l < HALO; l += NTHREADS) {
-      for (int q = f.B - 1; q >= 0; --q) sm[(3 + 2 * q) * HALO + l] = sm[(2 + q) * HALO + l];
-      float c = 0.f;
-      for (int q = 0; q < f.B; ++q) {
-        sm[(2 + 2 * q) * HALO + l] = c;
-        c += sm[(3 + 2 * q) * HALO + l];
+    // the table from the masses staged in rows 2 .. 1 + B
+    if (semi_apart(f.B)) {
+      constexpr int WS = semi_stride(HALO);
+      float *tab = reinterpret_cast<float *>(R4);
+      for (int l = threadIdx.x; l < HALO; l += NTHREADS) {
+        float c = 0.f;
+        for (int q = 0; q < f.B; ++q) {
+          const float m = sm[(2 + q) * HALO + l];
+          tab[2 * q * WS + l] = c;
+          tab[(2 * q + 1) * WS + l] = m;
+          c += m;
+        }
+        tab[2 * f.B * WS + l] = c;
+        tab[(2 * f.B + 1) * WS + l] = 0.f;
       }
-      sm[(2 + 2 * f.B) * HALO + l] = c;
-      sm[(3 + 2 * f.B) * HALO + l] = 0.f;
-    }
-    // what an absent neighbour reads, in the corner's rows (this thread built
-    // them)
-    if (threadIdx.x == 0) {
-      sm[2 * HALO] = 1.f;
-      sm[3 * HALO] = 0.f;
+      // what an absent neighbour reads, in the corner's rows (this thread
+      // built them)
+      if (threadIdx.x == 0) {
+        tab[0] = 1.f;
+        tab[WS] = 0.f;
+      }
+    } else {
+      // in place: the masses moved up to every other row (from the last: a
+      // mass moves to a row above those not yet moved), then the running sums
+      for (int l = threadIdx.x; l < HALO; l += NTHREADS) {
+        for (int q = f.B - 1; q >= 0; --q) sm[(3 + 2 * q) * HALO + l] = sm[(2 + q) * HALO + l];
+        float c = 0.f;
+        for (int q = 0; q < f.B; ++q) {
+          sm[(2 + 2 * q) * HALO + l] = c;
+          c += sm[(3 + 2 * q) * HALO + l];
+        }
+        sm[(2 + 2 * f.B) * HALO + l] = c;
+        sm[(3 + 2 * f.B) * HALO + l] = 0.f;
+      }
+      if (threadIdx.x == 0) {
+        sm[2 * HALO] = 1.f;
+        sm[3 * HALO] = 0.f;
+      }
     }
     __syncthreads();
   }
@@ -1247,14 +1273,14 @@ __device__ __forceinline__ void integrate_tile(const Field &f, int ty0, int tx0,
       const float lo1 = sm[l];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        nb[i].off = 2 * HALO + nl[i];
+        nb[i].off = nl[i];
         nb[i].T = T[i];
         if (!present[i]) {  // F = 1, G = T - F = 1 (semi_cdf)
           nb[i].kind = 0;
           nb[i].lam = 0.f;
           nb[i].ih = 0.f;
           nb[i].T = 2.f;
-          nb[i].off = 2 * HALO;
+          nb[i].off = 0;
           continue;
         }
         const float lo = sm[nl[i]], hi = sm[HALO + nl[i]];
@@ -1263,10 +1289,16 @@ __device__ __forceinline__ void integrate_tile(const Field &f, int ty0, int tx0,
         nb[i].ih = lo == hi ? 0.f : (float)f.B / (hi - lo);
       }
       const PhiloxKeys K(f.seed_lo, f.seed_hi);
-      if (!SADDLE || has_saddle)
-        semi_vertex<HALO, SADDLE>(sm, l, lo1, sm[HALO + l], nb, f.B, f.samples, K,
-                                  (uint32_t)((long long)gy * f.W + gx), f.field_id, sg, pmin,
-                                  pmax, psad);
+      const uint32_t vid = (uint32_t)((long long)gy * f.W + gx);
+      if (!SADDLE || has_saddle) {
+        if (semi_apart(f.B))
+          semi_vertex<semi_stride(HALO), SADDLE, true>(
+              reinterpret_cast<const float *>(R4), l, lo1, sm[HALO + l], nb, f.B, f.samples, K,
+              vid, f.field_id, sg, pmin, pmax, psad);
+        else
+          semi_vertex<HALO, SADDLE, false>(sm + 2 * HALO, l, lo1, sm[HALO + l], nb, f.B,
+                                           f.samples, K, vid, f.field_id, sg, pmin, pmax, psad);
+      }
       if (!SADDLE && f.boundary == 1 && k < 4) pmin = pmax = 0.f;
     } else if (MODEL == kUniform) {
       UniParams cp{sm[l], sm[HALO + l]}, nb[4];
