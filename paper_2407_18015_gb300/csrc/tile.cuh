@@ -608,41 +608,45 @@ __device__ __forceinline__ void cp_async_wait_all() {
 // that hold each (member, row) segment (see `load` in stage_members_tma for
 // the layout: column c of member m, row r at m PLANE + r kBoxW + c + d, d =
 // (address / 4) mod 4); the copies have landed for the whole CTA on return.
+// A thread owns one 16-byte block of one row and takes it of every GR-th
+// member.  Four members are a multiple of 16 bytes, so the blocks of members 4
+// apart are too, whatever H W mod 4 is: the thread keeps a pointer and a
+// verdict (whether the block holds a column that is read) for each of the up
+// to four residues, and a copy costs the copy and the pointer's advance
+// (addresses and bounds formed for every copy: 1021 x 1023 x 50, 5 bins 176 ->
+// 173 us, 64-field batch of mostly odd widths 3.03 -> 2.93 ms).
 template <int HY>
 __device__ __forceinline__ void box_copy_async(const Field &f, float *box, int k0, int nc,
                                                int ty0, int tx0, int ylim) {
-  constexpr int PLANE = HY * kBoxW;
-  const int N = f.N;
-  constexpr int SLOTS = NTHREADS / 5, DM = SLOTS / HY, DR = SLOTS % HY;
-  const int nseg = min(nc, N - k0) * HY;
-  if (threadIdx.x < SLOTS * 5) {
-    const int q = threadIdx.x % 5;
-    int sg = threadIdx.x / 5;
-    const int m = sg / HY;
-    int r = sg - m * HY;
+  constexpr int PLANE = HY * kBoxW, SLOTS = HY * (kBoxW / 4);
+  constexpr int GR = NTHREADS / SLOTS >= 2 ? 2 : 1, PH = 4 / GR;
+  static_assert(SLOTS <= NTHREADS, "a thread per block");
+  const int kn = min(nc, f.N - k0);
+  const int g = (int)threadIdx.x / SLOTS, s = (int)threadIdx.x % SLOTS;
+  const int r = s / (kBoxW / 4), j = 4 * (s % (kBoxW / 4));
+  const int gy = ty0 - 1 + r;
+  if (g < GR && (unsigned)gy < (unsigned)ylim) {
     // smem columns (before the shift d) that staged vertices read
     const int lo0 = max(tx0 - 1, 0) - tx0 + 4, hi0 = min(tx0 + 33, f.W) - tx0 + 4;
-    const uintptr_t rstep = (uintptr_t)f.W * 4u, pstep = (uintptr_t)f.plane * 4u;
-    uintptr_t a = reinterpret_cast<uintptr_t>(f.ens) +
-                  (uintptr_t)(((long long)(k0 + m) * f.plane +
-                               (long long)(ty0 - 1 + r) * f.W + (tx0 - 4)) * 4);
-    float *dst = box + m * PLANE + r * kBoxW + 8 * q;
-    for (; sg < nseg; sg += SLOTS) {
-      const int gy = ty0 - 1 + r;
-      if ((unsigned)gy < (unsigned)ylim) {
-        const int d = (int)(a >> 2) & 3;
-        const int lo = lo0 + d, hi = hi0 + d, j = 8 * q;
-        const uintptr_t cb = (a & ~(uintptr_t)15) + 32u * q;
-        if (j + 4 > lo && j < hi) cp_async16(dst, cb);
-        if (j + 8 > lo && j + 4 < hi) cp_async16(dst + 4, cb + 16);
-      }
-      r += DR;
-      a += DM * pstep + DR * rstep;
-      dst += DM * PLANE + DR * kBoxW;
-      if (r >= HY) {
-        r -= HY;
-        a += pstep - HY * rstep;
-        dst += PLANE - HY * kBoxW;
+    const uintptr_t pstep = (uintptr_t)f.plane * 4u;
+    const uintptr_t a = reinterpret_cast<uintptr_t>(f.ens) +
+                        (uintptr_t)(((long long)(k0 + g) * f.plane + (long long)gy * f.W +
+                                     (tx0 - 4)) * 4);
+    uintptr_t src[PH];
+    bool take[PH];
+#pragma unroll
+    for (int h = 0; h < PH; ++h) {
+      const uintptr_t ah = a + (uintptr_t)(h * GR) * pstep;
+      const int d = (int)(ah >> 2) & 3;
+      src[h] = (ah & ~(uintptr_t)15) + 4u * (unsigned)j;
+      take[h] = j + 4 > lo0 + d && j < hi0 + d;
+    }
+    float *dst = box + g * PLANE + r * kBoxW + j;
+    for (int m = g; m < kn; m += 4, dst += 4 * PLANE) {
+#pragma unroll
+      for (int h = 0; h < PH; ++h) {
+        if (take[h] && m + h * GR < kn) cp_async16(dst + h * GR * PLANE, src[h]);
+        src[h] += 4u * pstep;
       }
     }
   }
