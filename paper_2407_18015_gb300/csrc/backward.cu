@@ -907,7 +907,7 @@ __global__ void __launch_bounds__(NTHREADS, 2)
 // shared memory).  One running partial per neighbour, A = C(start of its bin)
 // + in-bin integral, scaled by the centre's weight, is stored as it is and
 // restarted at C; the rows carry 1/h, whose 0 also says that the walker is
-// not inside a bin.  2048 x 2048 vertices, 16 bins: 2.83 -> 2.26 ms (three
+// not inside a bin.  2048 x 2048 vertices, 16 bins: 2.83 -> 2.2 ms (three
 // Gauss-Legendre nodes, the partial in two parts and a width per walker
 // before).
 
@@ -919,7 +919,10 @@ __device__ __forceinline__ float rows_bin_width(float w, int B) {
 // One neighbour's crossing in the adjoint walk, without a branch: if its
 // next edge nx is at or below x1, store A (its partial of the bin it leaves)
 // at optr if it was inside a bin (r.y = 1/h, 0 outside), move optr to the
-// next bin's partial, restart A at C and read the next row into r.
+// next bin's partial, restart A at C and read the next row into r (in three
+// reads: a 16-byte one wants four adjacent registers, and the packed pairs'
+// halves were moved in and out of them: 3.34 -> 3.29 ms of the 2048 x 2048, 16
+// bin fit + forward + adjoint).
 template <unsigned stride>
 __device__ __forceinline__ void adj_cross(float nx, float x1, float *&optr, long long qs, float C,
                                           float &A, uint32_t &addr, float4 &r) {
@@ -930,7 +933,9 @@ __device__ __forceinline__ void adj_cross(float nx, float x1, float *&optr, long
       " @e st.global.f32 [%4], %6;\n"
       " @q add.s64 %4, %4, %9;\n"
       " @q mov.f32 %6, %10;\n"
-      " @q ld.shared.v4.f32 {%0, %1, %2, %3}, [%5];\n"
+      " @q ld.shared.f32 %0, [%5];\n"
+      " @q ld.shared.f32 %1, [%5 + 4];\n"
+      " @q ld.shared.v2.f32 {%2, %3}, [%5 + 8];\n"
       " @q add.u32 %5, %5, %11;\n}"
       : "+f"(r.x), "+f"(r.y), "+f"(r.z), "+f"(r.w), "+l"(optr), "+r"(addr), "+f"(A)
       : "f"(nx), "f"(x1), "l"(qs * (long long)sizeof(float)), "f"(C), "n"(stride)
