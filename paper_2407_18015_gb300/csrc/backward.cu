@@ -1146,9 +1146,31 @@ __device__ __forceinline__ void hist_adj_centre(const Field &f, const float *sm,
   if (sm[l] == sm[HALO + l]) {
     // a point-mass centre: the product of tails (global-memory path)
     hist_grad_vertex(f.params, plane, gi, ni, present, B, mirrored, wv, out, kAdjTV);
-  } else {
-    hist_adj_walk<HALO, RS>(sm, R4, l, nl, present, B, mirrored, wv, out, kAdjTV);
+    return;
   }
+  // A support that starts so far below the centre's that the finite edge of
+  // its end row lies inside the walk is not walked past its end: if it ends
+  // before the walk its survival is 0 there, and so is every partial; if it
+  // ends inside, it is too wide for the walk's frame (as a centre may be).
+  const float lo1 = sm[l], W1 = sm[HALO + l] - lo1;
+  float first = 0.f;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    if (present[i]) first = fminf(first, sm[nl[i]] - lo1);
+  if (first + kFar <= W1) {
+    bool below = false, inside = false;
+    for (int i = 0; i < 4; ++i) {
+      if (!present[i]) continue;
+      const float lam = sm[nl[i]] - lo1, e = lam + (sm[HALO + nl[i]] - sm[nl[i]]);
+      below |= e <= 0.f;
+      inside |= lam + kFar <= W1 && e <= W1;
+    }
+    if (below || inside) {
+      for (int q = 0; q < 5 * B; ++q) out[q * kAdjTV] = below ? 0.f : qnan();
+      return;
+    }
+  }
+  hist_adj_walk<HALO, RS>(sm, R4, l, nl, present, B, mirrored, wv, out, kAdjTV);
 }
 
 template <int RB>

@@ -1475,10 +1475,13 @@ __device__ __forceinline__ void lds64_cross(float nx, float x1, uint32_t &addr, 
 // T - S_k, slope_k, e_{k+1} - lo), with the tail S_k = T - (m_0 + ... +
 // m_{k-1}), slope_k = (S_k - S_{k+1}) / h (the bin's density, m_k / h, in
 // the mixture form) and e_{k+1} - lo = (k + 1) h (hi - lo for the last
-// edge).  Row B is (0, T, 0, kFar), beyond the support.  A point mass has
-// every row (0, T, 0, kFar): its one edge takes the survival from T to 0.
-// A walker reads a row only when it crosses an edge, at most B + 1 times,
-// so no row past B is ever read.
+// edge).  Row B is (0, T, 0, inf), beyond the support.  A point mass has
+// every row (0, T, 0, inf): its one edge takes the survival from T to 0.
+// A walker reads a row only when it crosses an edge, at most B + 1 times: no
+// edge follows row B, wherever the support starts (a finite last edge plus a
+// start below -2e38 could lie inside the walk), so no row past B is ever
+// read.  The adjoint's rows end with the finite kFar (it multiplies the
+// distance to the edge by 0) and it takes such starts out before its walk.
 __host__ __device__ constexpr int hist_r4_rows(int B) { return B + 1; }
 
 // Row stride of the per-bin rows of a halo of `halo` vertices, in float4:
@@ -1699,9 +1702,9 @@ __device__ __forceinline__ void hist_walk_pieces(const float4 *crow, int B, floa
   } else {
     // A turn's second piece may come after the walk's end: clamped to W1 it
     // has no width, and crosses nothing past the rows (the centre's next
-    // edge is then kFar, and a neighbour's are above W1 or were not yet
+    // edge is then infinite, and a neighbour's are above W1 or were not yet
     // crossed at it; without the clamp every walker beyond its support would
-    // "cross" kFar and read past its last row)
+    // "cross" its infinite edge and read past its last row)
 #pragma unroll 1
     for (int step = 0; step < max_steps && x0 < W1; step += 2) {
       piece(false);

@@ -375,7 +375,7 @@ template <int RS, int NB, bool FULL, bool ADJ = false, typename Mass>
 __device__ __forceinline__ void hist_rows_write(float4 *R, float a, float b, float t, int B,
                                                 Mass mass) {
   if constexpr (FULL) B = NB;
-  const float4 beyond = make_float4(0.f, ADJ ? 0.f : t, 0.f, kFar);
+  const float4 beyond = make_float4(0.f, ADJ ? 0.f : t, 0.f, ADJ ? kFar : __int_as_float(0x7f800000));
   R[B * RS] = beyond;
   if (a == b) {
     for (int k = 0; k < B; ++k) R[k * RS] = beyond;
