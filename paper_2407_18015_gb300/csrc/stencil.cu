@@ -187,7 +187,7 @@ struct HistTile {
 // SM: the walkers of eight neighbours need the registers.  Bound by
 // instruction issue; against tail tables in global memory, where every step
 // of every walker read its table through L1 whether it crossed or not: 1024
-// x 1024 x 20, 8 bins, eight neighbours 1.02 -> 0.52 ms, fit included.
+// x 1024 x 20, 8 bins, eight neighbours 1.02 -> 0.50 ms, fit included.
 template <int ST, int RB, int MODE>
 __global__ void __launch_bounds__(NTHREADS, 2) stencil_hist_kernel(StencilField f, int tiles_x,
                                                                    int tiles_y) {

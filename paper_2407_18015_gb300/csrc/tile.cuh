@@ -839,7 +839,7 @@ __device__ __forceinline__ bool stage_members_tma(const Field &f, float *sm, flo
           s2[p].add(d * d);
         }
       };
-      box_members<PLANE, ASYNC>(col, kn, sh, pl, MemberPairs{
+      const MemberPairs reduce{
           [&](float v1, float v2) {
             mn[p] = fmin3_nan(mn[p], v1, v2);
             mx[p] = fmax3_nan(mx[p], v1, v2);
@@ -850,7 +850,18 @@ __device__ __forceinline__ bool stage_members_tma(const Field &f, float *sm, flo
             mn[p] = fmin_nan(mn[p], v);
             mx[p] = fmax_nan(mx[p], v);
             add(v);
-          }});
+          }};
+      if constexpr (!EP && !ASYNC) {
+        // minima and maxima alone: eight members to a turn, and member 0
+        // not again (uniform, 2048 x 2048 x 20: 111.7 -> 106.4 us against
+        // box_members; 8 bins, 1024 x 1024 x 20: 143.3 -> 141.2)
+        int k = k0 == 0 ? 1 : 0;
+#pragma unroll 4
+        for (; k + 1 < kn; k += 2) reduce(col[k * PLANE], col[(k + 1) * PLANE]);
+        if (k < kn) reduce(col[k * PLANE]);
+      } else {
+        box_members<PLANE, ASYNC>(col, kn, sh, pl, reduce);
+      }
     }
     __syncthreads();
   }
