@@ -1435,8 +1435,8 @@ __device__ __forceinline__ void hist_walk(const float *S0, int coff, int B, floa
 
 // Crossing step of a walker over shared-memory rows: if nx <= x1, read the
 // 16-byte row at addr into v and advance addr by `stride` bytes; else leave
-// both.  One comparison, one predicated read and one predicated add, no
-// branch.  addr: a shared-state-space address.
+// both.  One comparison, predicated reads and a predicated add, no branch.
+// addr: a shared-state-space address.
 template <unsigned stride>
 __device__ __forceinline__ void lds128_cross(float nx, float x1, uint32_t &addr, float4 &v) {
   asm("{\n .reg .pred q;\n setp.le.f32 q, %5, %6;\n"
@@ -1445,12 +1445,22 @@ __device__ __forceinline__ void lds128_cross(float nx, float x1, uint32_t &addr,
       : "+f"(v.x), "+f"(v.y), "+f"(v.z), "+f"(v.w), "+r"(addr)
       : "f"(nx), "f"(x1), "n"(stride));
 }
+// The same in two 8-byte reads: a 16-byte one wants four adjacent registers,
+// and the packed arithmetic of a walk unrolled twice moves between pairs (1024
+// x 1024 vertices from parameters, 16 bins, both types 263 -> 254 us).
+template <unsigned stride>
+__device__ __forceinline__ void lds2x64_cross(float nx, float x1, uint32_t &addr, float4 &v) {
+  asm("{\n .reg .pred q;\n setp.le.f32 q, %5, %6;\n"
+      " @q ld.shared.v2.f32 {%0, %1}, [%4];\n"
+      " @q ld.shared.v2.f32 {%2, %3}, [%4 + 8];\n"
+      " @q add.u32 %4, %4, %7;\n}"
+      : "+f"(v.x), "+f"(v.y), "+f"(v.z), "+f"(v.w), "+r"(addr)
+      : "f"(nx), "f"(x1), "n"(stride));
+}
 // The same for a walk of one type: of the row's (G, F, slope, next edge) only
-// that type's value (at byte OFF) and the last two are read, by two reads.  A
-// 16-byte read wants its four registers adjacent, and the walk's arithmetic
-// then moved the value in and out of them: 12 of 66 instructions per step
-// (1024 x 1024 vertices from parameters, 8 bins 118 -> 108 us, 16 bins 223 ->
-// 217).
+// that type's value (at byte OFF) and the last two are read (1024 x 1024
+// vertices from parameters, against the 16-byte read: 8 bins 118 -> 108 us, 16
+// bins 223 -> 217).
 template <unsigned stride, unsigned OFF>
 __device__ __forceinline__ void lds_cross1(float nx, float x1, uint32_t &addr, float &g, float &z,
                                            float &w) {
@@ -1497,8 +1507,8 @@ __host__ __device__ constexpr int hist_r4_stride(int halo) { return (halo + 7) &
 // slope_k per unit of x; beyond it (0, T).  The walker holds the row of its
 // current segment, (G, F, slope, next edge - lo) with G and F taken at the
 // walk's current position, advances G and F by the step length and,
-// crossing an edge, lets one predicated 16-byte read replace the whole state
-// with the next row, whose (S_k, T - S_k) are the exact values at that edge
+// crossing an edge, lets predicated reads replace the whole state with the
+// next row, whose (S_k, T - S_k) are the exact values at that edge
 // (which also carries the jump of a point mass).  An absent neighbour is the
 // constant G = F = 1 that never reaches an edge.
 struct HistRowWalker {
@@ -1583,49 +1593,63 @@ __device__ __forceinline__ float fmin5(float a, float b, float c, float d, float
   return r;
 }
 
-// A walker's crossing in a walk of mode MODE.
-template <int RS, int MODE>
+// A walker's crossing in a walk of mode MODE; QUAD: rows read whole.
+template <int RS, int MODE, bool QUAD = false>
 __device__ __forceinline__ void walker_cross(float nx, float x1, HistRowWalker &n) {
   constexpr unsigned stride = (unsigned)(RS * 16);
   if constexpr (MODE == kWalkMin) lds_cross1<stride, 0>(nx, x1, n.addr, n.r.x, n.r.z, n.r.w);
   else if constexpr (MODE == kWalkMax) lds_cross1<stride, 4>(nx, x1, n.addr, n.r.y, n.r.z, n.r.w);
-  else lds128_cross<stride>(nx, x1, n.addr, n.r);
+  else if constexpr (QUAD) lds128_cross<stride>(nx, x1, n.addr, n.r);
+  else lds2x64_cross<stride>(nx, x1, n.addr, n.r);
+}
+
+// Mean over a piece of the product of four linear factors given by their left
+// and right values, taken in two pairs: with b0 = L0 L1, b2 = R0 R1, b1 = L0 R1
+// + R0 L1 (the pair's quadratic in the Bernstein basis, middle coefficient
+// doubled) and c0, c1, c2 likewise for factors 2 and 3 it is
+//   (b0 c0 + b2 c2) / 5 + ((b0 + b2) c1 + b1 (c0 + c2)) / 20
+//   + (b0 c2 + b2 c0 + b1 c1) / 30,
+// every term a product of non-negative end values.
+template <typename O, typename V>
+__device__ __forceinline__ V bern_mean4_pairs(const V *L, const V *R) {
+  const V b0 = O::mul(L[0], L[1]), b2 = O::mul(R[0], R[1]);
+  const V b1 = O::fma(L[0], R[1], O::mul(R[0], L[1]));
+  const V c0 = O::mul(L[2], L[3]), c2 = O::mul(R[2], R[3]);
+  const V c1 = O::fma(L[2], R[3], O::mul(R[2], L[3]));
+  const V t1 = O::fma(b0, c0, O::mul(b2, c2));
+  const V t2 = O::fma(O::add(b0, b2), c1, O::mul(b1, O::add(c0, c2)));
+  const V t3 = O::fma(b0, c2, O::fma(b2, c0, O::mul(b1, c1)));
+  return O::fma(O::all(0.2f), t1, O::fma(O::all(0.05f), t2, O::mul(O::all(1.f / 30.f), t3)));
 }
 
 // The probabilities of a non-degenerate histogram centre in one walk over
 // [0, W1] (local frame at lo1; the centre's rows from crow): all bin edges of
 // the centre and of the four neighbours are merged in increasing order; on
 // each piece the centre pdf is the constant m_j / h1 and each factor is
-// linear, f_i = l_i + D_i t, so the product f is a quartic in t in [0, 1] and
-// Simpson's rule with its fourth-order term is exact:
-//   int f = (f(0) + 4 f(1/2) + f(1)) / 6 - D_0 D_1 D_2 D_3 / 120
-// (for t^4: 1/5 = 5/24 - 1/120).  The values are products of non-negative
-// factors and the correction is at most a quarter of the result (t^2 (1 -
-// t)^2), so nothing cancels.  The product D_0..D_3 has the same sign in the
-// two products of a mode (each D changes sign between G and F).  f(0) is the
-// previous piece's f(1): with CARRY it is handed on; a point-mass neighbour's
-// survival jumps at its position, so those walks form it anew.  Beyond a
-// neighbour's support its survival is 0, before it its CDF is 0, so the
-// integrals run over the centre's whole support.  Every lane executes the
-// same instructions on every step; only the row reads of the crossings are
-// predicated.
+// linear, so the piece's integral is the Bernstein mean of the factors' end
+// values.  The left values are the walkers' current rows': a row read at a
+// crossing brings the exact tails of its edge, where the previous piece's right
+// value is off by the rounding of the edges' positions against the bin's width
+// (all of a bin's mass where its edges round together; carried on, it would
+// enter the whole next piece).  Beyond a neighbour's support its survival is
+// 0, before it its CDF is 0, so the integrals run over the centre's whole
+// support.  Every lane executes the same instructions on every step; only the
+// row reads of the crossings are predicated.
 //
-// Bound by instruction issue (70-80 % of the slots) and the FP32 pipe, which
-// a packed instruction takes for two cycles.  With both products: (G, F) at
-// the middle and the end of a piece are one packed multiply-add each, from
-// the row's slope in both halves, and stay where the row read puts them: 60
-// instructions per step (90 with the Bernstein mean of end values formed by
-// scalar multiply-adds).  With one product the arithmetic is scalar, half the
-// FP32 pipe's work, and two pieces are taken per turn (no test between them;
-// the second one is clamped to the walk's end, where no edge is left to
-// cross).  Walks over 1024 x 1024 vertices from parameters: 8 bins, both
-// types 167 -> 129 us, one type 167 -> 124; 16 bins 330 -> 264 and 330 ->
-// 234.
+// Bound by instruction issue and the FP32 pipe, which a packed instruction
+// takes for two cycles.  With both products (G, F) move to the end of a piece
+// by one packed multiply-add, from the row's slope in both halves; with one
+// the arithmetic is scalar, half the FP32 pipe's work.  Two pieces per turn, no
+// test between them: the new values' registers of the first are the old ones
+// of the second, without moves.  Walks over 1024 x 1024 vertices from
+// parameters: 8 bins, both types 128 us (137 with scalar multiply-adds and
+// 16-byte row reads, 134 with one piece per turn), one type 108; 16 bins 254
+// (274, 270) and 220.
 // Both: (pmin, pmax) = (int pdf prod G, int pdf prod F); one type: its own
 // output alone.  Saddle: (pmin, pmax) = (t1, t2) with factor i = G_i if
 // sg[i] > 0 else F_i for t1, and the other one for t2 (absent neighbours are
 // 1 in both).
-template <int RS, int MODE, bool CARRY>
+template <int RS, int MODE>
 __device__ __forceinline__ void hist_walk_pieces(const float4 *crow, int B, float W1,
                                                  HistRowWalker *nw, float &pmin, float &pmax,
                                                  const int *sg) {
@@ -1646,98 +1670,68 @@ __device__ __forceinline__ void hist_walk_pieces(const float4 *crow, int B, floa
     else if constexpr (MODE == kWalkMin) return g;
     else return ff;
   };
-  auto prod4 = [&](const V *a) { return O::mul(O::mul(a[0], a[1]), O::mul(a[2], a[3])); };
-  auto left = [&]() {
-    V L[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) L[i] = factor(i, nw[i].r.x, nw[i].r.y);
-    return prod4(L);
-  };
-  V acc = O::all(0.f), f0 = left();
+  V acc = O::all(0.f);
   float x0 = 0.f;
   auto piece = [&](bool clamp) {
     const float e[4] = {nw[0].nx(), nw[1].nx(), nw[2].nx(), nw[3].nx()};
     float x1 = fmin5(e[0], e[1], e[2], e[3], dc.y);
     if (clamp) x1 = fminf(x1, W1);
-    const float d = x1 - x0, hd = 0.5f * d;
-    const float dd = __fmul_rn(
-        __fmul_rn(__fmul_rn(nw[0].r.z, d), __fmul_rn(nw[1].r.z, d)),
-        __fmul_rn(__fmul_rn(nw[2].r.z, d), __fmul_rn(nw[3].r.z, d)));
-    if constexpr (!CARRY) f0 = left();
-    V M[4], R[4];  // middle and right values; the walkers move to x1
+    const float d = x1 - x0;
+    V L[4], R[4];  // left and right values; the walkers move to x1
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       float4 &r = nw[i].r;
+      L[i] = factor(i, r.x, r.y);
       if constexpr (O::two) {
-        const float2 zz = make_float2(r.z, r.z), l = make_float2(r.x, r.y);
-        const float2 m = __ffma2_rn(zz, make_float2(-hd, hd), l);
-        const float2 v = __ffma2_rn(zz, make_float2(-d, d), l);
+        const float2 v = __ffma2_rn(make_float2(r.z, r.z), make_float2(-d, d),
+                                    make_float2(r.x, r.y));
         r.x = v.x;
         r.y = v.y;
-        M[i] = factor(i, m.x, m.y);
-        R[i] = factor(i, v.x, v.y);
       } else {
         float &l = MODE == kWalkMin ? r.x : r.y;
-        M[i] = __fmaf_rn(r.z, MODE == kWalkMin ? -hd : hd, l);
         l = __fmaf_rn(r.z, MODE == kWalkMin ? -d : d, l);
-        R[i] = l;
       }
+      R[i] = factor(i, r.x, r.y);
     }
-    const V e1 = prod4(R), em = prod4(M);
-    // six times the mean of the product over the piece
-    const V m6 = O::fma(O::all(-0.05f), O::all(dd), O::fma(O::all(4.f), em, O::add(f0, e1)));
-    acc = O::fma(O::all(__fmul_rn(d, dc.x)), m6, acc);
-    f0 = e1;
+    acc = O::fma(O::all(__fmul_rn(d, dc.x)), bern_mean4_pairs<O>(L, R), acc);
 #pragma unroll
     for (int i = 0; i < 4; ++i) walker_cross<RS, MODE>(e[i], x1, nw[i]);
     lds64_cross<(unsigned)(RS * 16)>(dc.y, x1, addr_c, dc);
     x0 = x1;
   };
+  // A turn's second piece may come after the walk's end: clamped to W1 it has
+  // no width, and crosses nothing past the rows (the centre's next edge is then
+  // infinite, and a neighbour's are above W1 or were not yet crossed at it;
+  // without the clamp every walker beyond its support would "cross" its
+  // infinite edge and read past its last row)
   const int max_steps = 5 * (B + 1) + 4;
+#pragma unroll 1
+  for (int step = 0; step < max_steps && x0 < W1; step += 2) {
+    piece(false);
+    piece(true);
+  }
   if constexpr (O::two) {
-#pragma unroll 1
-    for (int step = 0; step < max_steps && x0 < W1; ++step) piece(false);
-    pmin = fmaxf(__fmul_rn(acc.x, 1.f / 6.f), 0.f);
-    pmax = fmaxf(__fmul_rn(acc.y, 1.f / 6.f), 0.f);
+    pmin = fmaxf(acc.x, 0.f);
+    pmax = fmaxf(acc.y, 0.f);
   } else {
-    // A turn's second piece may come after the walk's end: clamped to W1 it
-    // has no width, and crosses nothing past the rows (the centre's next
-    // edge is then infinite, and a neighbour's are above W1 or were not yet
-    // crossed at it; without the clamp every walker beyond its support would
-    // "cross" its infinite edge and read past its last row)
-#pragma unroll 1
-    for (int step = 0; step < max_steps && x0 < W1; step += 2) {
-      piece(false);
-      piece(true);
-    }
-    (MODE == kWalkMin ? pmin : pmax) = fmaxf(__fmul_rn(acc, 1.f / 6.f), 0.f);
+    (MODE == kWalkMin ? pmin : pmax) = fmaxf(acc, 0.f);
   }
 }
 
-// hist_walk_pieces for the wanted types; point_mass: whether a present
-// neighbour is one (the lanes with one then walk apart from the others).
-// One type alone gives the same bits as in the walk of both.
+// hist_walk_pieces for the wanted types.  One type alone gives the same bits
+// as in the walk of both.
 template <int RS, bool SADDLE = false>
 __device__ __forceinline__ void hist_walk_rows(const float4 *crow, int B, float W1,
-                                               HistRowWalker *nw, bool point_mass,
-                                               unsigned types, float &pmin, float &pmax,
-                                               const int *sg = nullptr) {
+                                               HistRowWalker *nw, unsigned types, float &pmin,
+                                               float &pmax, const int *sg = nullptr) {
   if (!(W1 <= 1e38f)) {
     pmin = pmax = __int_as_float(0x7fc00000);
     return;
   }
-  if constexpr (SADDLE) {
-    if (!point_mass) hist_walk_pieces<RS, kWalkSaddle, true>(crow, B, W1, nw, pmin, pmax, sg);
-    else hist_walk_pieces<RS, kWalkSaddle, false>(crow, B, W1, nw, pmin, pmax, sg);
-  } else if (point_mass) {
-    hist_walk_pieces<RS, kWalkBoth, false>(crow, B, W1, nw, pmin, pmax, sg);
-  } else if (types == kMin) {
-    hist_walk_pieces<RS, kWalkMin, true>(crow, B, W1, nw, pmin, pmax, sg);
-  } else if (types == kMax) {
-    hist_walk_pieces<RS, kWalkMax, true>(crow, B, W1, nw, pmin, pmax, sg);
-  } else {
-    hist_walk_pieces<RS, kWalkBoth, true>(crow, B, W1, nw, pmin, pmax, sg);
-  }
+  if constexpr (SADDLE) hist_walk_pieces<RS, kWalkSaddle>(crow, B, W1, nw, pmin, pmax, sg);
+  else if (types == kMin) hist_walk_pieces<RS, kWalkMin>(crow, B, W1, nw, pmin, pmax, sg);
+  else if (types == kMax) hist_walk_pieces<RS, kWalkMax>(crow, B, W1, nw, pmin, pmax, sg);
+  else hist_walk_pieces<RS, kWalkBoth>(crow, B, W1, nw, pmin, pmax, sg);
 }
 
 // survival and CDF of a histogram neighbour (tail table S, total T) at a

@@ -328,7 +328,6 @@ __device__ __forceinline__ void integrate3(const Field3 &F, int ty0, int tx0, co
       }
     } else if (!zero_b) {
       HistRowWalker nw[4];
-      bool pm = false;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         HistRowWalker &h = nw[i];
@@ -337,11 +336,10 @@ __device__ __forceinline__ void integrate3(const Field3 &F, int ty0, int tx0, co
           continue;
         }
         const float lo = smh[nl[i]], hi = smh[HALO + nl[i]];
-        pm |= lo == hi;
         h.init(R4 + nl[i], lo - lo1, T[i]);
         h.seek0<RS>(R4 + nl[i], B, lo == hi ? 0.f : (hi - lo) * (1.f / (float)B));
       }
-      hist_walk_rows<RS>(R4 + l, B, hi1 - lo1, nw, pm, f.cptypes, pmin, pmax);
+      hist_walk_rows<RS>(R4 + l, B, hi1 - lo1, nw, f.cptypes, pmin, pmax);
     }
     put(2, pmin, pmax, st);
   }

@@ -479,7 +479,7 @@ __device__ __forceinline__ void hist_walk_rows_k(const float4 *crow, int B, floa
     }
     acc = O::fma(O::all(__fmul_rn(d, dc.x)), linear_mean_k<K, O>(m, D), acc);
 #pragma unroll
-    for (int i = 0; i < K; ++i) walker_cross<RS, MODE>(e[i], x1, nw[i]);
+    for (int i = 0; i < K; ++i) walker_cross<RS, MODE, true>(e[i], x1, nw[i]);
     lds64_cross<(unsigned)(RS * 16)>(dc.y, x1, addr_c, dc);
     x0 = x1;
   }

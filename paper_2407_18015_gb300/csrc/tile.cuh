@@ -1371,7 +1371,6 @@ __device__ __forceinline__ void integrate_tile(const Field &f, int ty0, int tx0,
         if (do_sad) psad = t1 + t2;
       } else if ((do_mm || do_sad) && ROWS) {
         HistRowWalker nw[4];
-        bool pm = false;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           HistRowWalker &h = nw[i];
@@ -1380,7 +1379,6 @@ __device__ __forceinline__ void integrate_tile(const Field &f, int ty0, int tx0,
             continue;
           }
           const float lo = sm[nl[i]], hi = sm[HALO + nl[i]];
-          pm |= lo == hi;
           h.init(R4 + nl[i], lo - lo1, T[i]);
           // the bin width only estimates how many edges lie below 0 (seek0
           // checks the estimate against the edges of the rows), so it need
@@ -1388,10 +1386,10 @@ __device__ __forceinline__ void integrate_tile(const Field &f, int ty0, int tx0,
           h.seek0<RS>(R4 + nl[i], B, lo == hi ? 0.f : (hi - lo) * (1.f / (float)B));
         }
         if constexpr (!SADDLE) {
-          hist_walk_rows<RS>(R4 + l, B, hi1 - lo1, nw, pm, f.cptypes, pmin, pmax);
+          hist_walk_rows<RS>(R4 + l, B, hi1 - lo1, nw, f.cptypes, pmin, pmax);
         } else {
           float t1, t2;
-          hist_walk_rows<RS, true>(R4 + l, B, hi1 - lo1, nw, pm, 0u, t1, t2, sg);
+          hist_walk_rows<RS, true>(R4 + l, B, hi1 - lo1, nw, 0u, t1, t2, sg);
           psad = t1 + t2;
         }
       } else if ((do_mm || do_sad) && !ROWS) {
