@@ -374,7 +374,7 @@ __device__ __forceinline__ void epan_grad_vertex(float m1, float w1, const float
       if (wn[i] == 0.f) {
         R = fminf(R, dn);
       } else {
-        al[i] = dn - wn[i]; d[i] = dn; iw[i] = 1.f / wn[i];
+        al[i] = dn - wn[i]; d[i] = dn; iw[i] = rcp_held(1.f / wn[i]);
         R = fminf(R, dn + wn[i]);
       }
     }
@@ -401,7 +401,7 @@ __device__ __forceinline__ void epan_grad_vertex(float m1, float w1, const float
       gw *= -0.75f * iw1 * iw1;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const float c = (0.75f * iw1) * (0.75f * pay[1][i]);
+        const float c = rcp_held((0.75f * iw1) * (0.75f * pay[1][i]));
         am[i] *= c;
         aw[i] *= c;
       }

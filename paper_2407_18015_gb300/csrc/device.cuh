@@ -51,6 +51,10 @@ constexpr float kFar = 3.0e38f;  // "never starts" breakpoint (finite: 0*kFar = 
 // sequence): support widths and bin widths only.
 __device__ __forceinline__ float frcp(float x) { return __fdividef(1.0f, x); }
 
+// A reciprocal held at the largest float: 1 / w of a subnormal width is beyond
+// it, and times a piece of zero width it has to be 0.
+__device__ __forceinline__ float rcp_held(float r) { return fminf(r, 3.402823466e38f); }
+
 // NaN-propagating minimum / maximum (a NaN input gives NaN; otherwise the
 // same value as fminf / fmaxf): a running min and max over members then
 // flag a non-finite member by themselves (NaN: both NaN; +Inf: the max;
@@ -709,7 +713,7 @@ __device__ __forceinline__ void epan_vertex(EpanParams c, const EpanParams *nb,
           al[i] = kFar; d[i] = kFar; iw[i] = 0.f;
           R = fminf(R, dn);
         } else {
-          al[i] = dn - wn; d[i] = dn; iw[i] = frcp(wn);
+          al[i] = dn - wn; d[i] = dn; iw[i] = rcp_held(frcp(wn));
           R = fminf(R, dn + wn);
         }
       } else {
@@ -729,7 +733,7 @@ __device__ __forceinline__ void epan_vertex(EpanParams c, const EpanParams *nb,
           al[i] = kFar; d[i] = kFar; iw[i] = 0.f;
           R = fminf(R, dn);
         } else {
-          al[i] = dn - wn; d[i] = dn; iw[i] = frcp(wn);
+          al[i] = dn - wn; d[i] = dn; iw[i] = rcp_held(frcp(wn));
           R = fminf(R, dn + wn);
         }
       } else {
@@ -1011,10 +1015,10 @@ __device__ __forceinline__ float epan_mixed(EpanParams c, const EpanParams *nb, 
     const float dn = nb[i].m - c.m, wn = nb[i].w;
     if (sg[i] > 0) {
       R = fminf(R, dn + wn);
-      if (wn > 0.f) { bp[i] = dn - wn; d[i] = dn; iw[i] = frcp(wn); }
+      if (wn > 0.f) { bp[i] = dn - wn; d[i] = dn; iw[i] = rcp_held(frcp(wn)); }
     } else {
       L = fmaxf(L, dn - wn);
-      if (wn > 0.f) { bp[i] = dn + wn; d[i] = dn; iw[i] = -frcp(wn); }
+      if (wn > 0.f) { bp[i] = dn + wn; d[i] = dn; iw[i] = -rcp_held(frcp(wn)); }
     }
   }
   if (!(R > L)) return 0.f;

@@ -268,7 +268,7 @@ __device__ __forceinline__ void epan_vertex_k(EpanParams c, const EpanParams *nb
       if (wn == 0.f) {  // point mass: survival 1 below it, and it caps R
         R = fminf(R, dn);
       } else {
-        al[i] = dn - wn; d[i] = dn; iw[i] = frcp(wn);
+        al[i] = dn - wn; d[i] = dn; iw[i] = rcp_held(frcp(wn));
         R = fminf(R, dn + wn);
       }
     }
