@@ -904,41 +904,44 @@ __global__ void __launch_bounds__(NTHREADS, 2)
 // a neighbour leaves a bin (or the centre leaves one of its own).
 //
 // Bound by instruction issue and the FP32 pipe at two CTAs per SM (the rows'
-// shared memory).  One running partial per neighbour, A = C(start of its bin)
-// + in-bin integral, scaled by the centre's weight, is stored as it is and
-// restarted at C; the rows carry 1/h, whose 0 also says that the walker is
-// not inside a bin.  2048 x 2048 vertices, 16 bins: 2.83 -> 2.2 ms (three
-// Gauss-Legendre nodes, the partial in two parts and a width per walker
-// before).
+// shared memory).  The running sums carry the centre's weight, so that a
+// partial, C at the start of the bin plus the in-bin integral, is stored as it
+// is.  The two stay apart until then: one running sum of both is 3 % faster
+// (2.22 ms) but rounds, or loses, each piece at the size of C.  The rows carry
+// 1/h, whose 0 also says that the walker is not inside a bin.  2048 x 2048
+// vertices, 16 bins: 2.88 -> 2.29 ms (three Gauss-Legendre nodes and a width
+// per walker before).
 
-// the bin width of the rows of a support of width w (as hist_rows_build)
+// the bin width of the rows of a support of width w (as hist_rows_write)
 __device__ __forceinline__ float rows_bin_width(float w, int B) {
   return (B & (B - 1)) == 0 ? w * (1.f / (float)B) : w / (float)B;
 }
 
 // One neighbour's crossing in the adjoint walk, without a branch: if its
-// next edge nx is at or below x1, store A (its partial of the bin it leaves)
-// at optr if it was inside a bin (r.y = 1/h, 0 outside), move optr to the
-// next bin's partial, restart A at C and read the next row into r (in three
+// next edge nx is at or below x1, store val (its partial of the bin it leaves)
+// at optr if it was inside a bin (r.y = 1/h, 0 outside), move optr to the next
+// bin's partial, restart Cs = C and I = 0 and read the next row into r (in three
 // reads: a 16-byte one wants four adjacent registers, and the packed pairs'
 // halves were moved in and out of them: 3.34 -> 3.29 ms of the 2048 x 2048, 16
-// bin fit + forward + adjoint).
+// bin fit + forward + adjoint, then with one sum).
 template <unsigned stride>
-__device__ __forceinline__ void adj_cross(float nx, float x1, float *&optr, long long qs, float C,
-                                          float &A, uint32_t &addr, float4 &r) {
+__device__ __forceinline__ void adj_cross(float nx, float x1, float *&optr, long long qs, float val,
+                                          float C, float &Cs, float &I, uint32_t &addr,
+                                          float4 &r) {
   asm volatile(
       "{\n .reg .pred q, e;\n"
-      " setp.le.f32 q, %7, %8;\n"
+      " setp.le.f32 q, %8, %9;\n"
       " setp.ne.and.f32 e, %1, 0f00000000, q;\n"
-      " @e st.global.f32 [%4], %6;\n"
-      " @q add.s64 %4, %4, %9;\n"
-      " @q mov.f32 %6, %10;\n"
+      " @e st.global.f32 [%4], %13;\n"
+      " @q add.s64 %4, %4, %10;\n"
+      " @q mov.f32 %6, %11;\n"
+      " @q mov.f32 %7, 0f00000000;\n"
       " @q ld.shared.f32 %0, [%5];\n"
       " @q ld.shared.f32 %1, [%5 + 4];\n"
       " @q ld.shared.v2.f32 {%2, %3}, [%5 + 8];\n"
-      " @q add.u32 %5, %5, %11;\n}"
-      : "+f"(r.x), "+f"(r.y), "+f"(r.z), "+f"(r.w), "+l"(optr), "+r"(addr), "+f"(A)
-      : "f"(nx), "f"(x1), "l"(qs * (long long)sizeof(float)), "f"(C), "n"(stride)
+      " @q add.u32 %5, %5, %12;\n}"
+      : "+f"(r.x), "+f"(r.y), "+f"(r.z), "+f"(r.w), "+l"(optr), "+r"(addr), "+f"(Cs), "+f"(I)
+      : "f"(nx), "f"(x1), "l"(qs * (long long)sizeof(float)), "f"(C), "n"(stride), "f"(val)
       : "memory");
 }
 
@@ -981,12 +984,13 @@ __device__ __forceinline__ void hist_adj_walk(const float *sm, const float4 *R4,
     return;
   }
   HistRowWalker nw[4];
-  // per neighbour: C = int_0^x pdf_1 LOO, A = C at the start of its current
-  // bin + the in-bin integral of that bin (both times wv); its bin (-1 before
+  // per neighbour: C = int_0^x pdf_1 LOO, Cs = C at the start of its current
+  // bin, I = the in-bin integral of that bin (all times wv; kept apart, since a
+  // sum of both would round every piece at the size of C); its bin (-1 before
   // the support, B beyond; a point mass moves from -1 to 0 at its position
   // and stays there) follows from the address of its next row
   float2 C02 = {0.f, 0.f}, C13 = {0.f, 0.f};
-  float A[4] = {0.f, 0.f, 0.f, 0.f};
+  float Cs[4] = {0.f, 0.f, 0.f, 0.f}, I[4] = {0.f, 0.f, 0.f, 0.f};
   float *optr[4];  // the partial of neighbour i's current bin (used inside a bin only)
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -1044,28 +1048,28 @@ __device__ __forceinline__ void hist_adj_walk(const float *sm, const float4 *R4,
     const float2 b = __ffma2_rn(mA, DB, __fmul2_rn(mB, DA)), b3 = __fmul2_rn(b, third);
     const float2 U = __ffma2_rn(g, third, p), V = __ffma2_rn(p, third, __fmul2_rn(g, fifth));
     own = fmaf(d * wvh, fmaf(p.x, U.y, fmaf(g.x, V.y, b.x * b3.y)), own);
-    // the other pair's, times the centre's density, weight and the width
+    // leave-one-out integrals of (0, 2) from the factors (1, 3) and the other
+    // pair's, and back; then the centre's density, weight and the width
     const float a = (d * dc.x) * wv;
     const float2 aa = make_float2(a, a);
-    const float2 Uo = __fmul2_rn(aa, make_float2(U.y, U.x));
-    const float2 Vo = __fmul2_rn(aa, make_float2(V.y, V.x));
-    const float2 bo = __fmul2_rn(aa, make_float2(b3.y, b3.x));
-    // leave-one-out integrals of (0, 2) from the factors (1, 3), and back
+    const float2 Uo = make_float2(U.y, U.x), Vo = make_float2(V.y, V.x);
+    const float2 bo = make_float2(b3.y, b3.x);
     const float2 sA = __ffma2_rn(mB, Uo, __fmul2_rn(DB, bo));
     const float2 sB = __ffma2_rn(mA, Uo, __fmul2_rn(DA, bo));
     const float2 tA = __ffma2_rn(mB, bo, __fmul2_rn(DB, Vo));
     const float2 tB = __ffma2_rn(mA, bo, __fmul2_rn(DA, Vo));
-    C02 = __fadd2_rn(C02, sA);
-    C13 = __fadd2_rn(C13, sB);
-    const float2 a02 = __ffma2_rn(vA, tA, __ffma2_rn(wA, sA, make_float2(A[0], A[2])));
-    const float2 a13 = __ffma2_rn(vB, tB, __ffma2_rn(wB, sB, make_float2(A[1], A[3])));
-    A[0] = a02.x; A[2] = a02.y; A[1] = a13.x; A[3] = a13.y;
+    C02 = __ffma2_rn(aa, sA, C02);
+    C13 = __ffma2_rn(aa, sB, C13);
+    const float2 i02 = __ffma2_rn(aa, __ffma2_rn(vA, tA, __fmul2_rn(wA, sA)), make_float2(I[0], I[2]));
+    const float2 i13 = __ffma2_rn(aa, __ffma2_rn(vB, tB, __fmul2_rn(wB, sB)), make_float2(I[1], I[3]));
+    I[0] = i02.x; I[2] = i02.y; I[1] = i13.x; I[3] = i13.y;
     const float C[4] = {C02.x, C13.x, C02.y, C13.y};
     // crossings: a neighbour leaving bin k stores its partial
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       nw[i].r.x = fmaf(-nw[i].r.z, d, nw[i].r.x);
-      adj_cross<(unsigned)(RS * 16)>(e[i], x1, optr[i], qstride, C[i], A[i], nw[i].addr, nw[i].r);
+      adj_cross<(unsigned)(RS * 16)>(e[i], x1, optr[i], qstride, Cs[i] + I[i], C[i], Cs[i], I[i],
+                                     nw[i].addr, nw[i].r);
     }
     adj_cross_centre<(unsigned)(RS * 16)>(x1, optr_c, qstride, own, addr_c, dc);
     x0 = x1;
@@ -1081,11 +1085,11 @@ __device__ __forceinline__ void hist_adj_walk(const float *sm, const float4 *R4,
     const uint32_t row0 = static_cast<uint32_t>(__cvta_generic_to_shared(R4 + nl[i]));
     const int kb = (int)((nw[i].addr - row0) / (uint32_t)(RS * 16)) - 1;
     const bool pm = sm[nl[i]] == sm[HALO + nl[i]];
-    if (kb >= 0 && kb < B) *out(1 + i, kb) = A[i];
+    if (kb >= 0 && kb < B) *out(1 + i, kb) = Cs[i] + I[i];
     // bins entirely above the walk: their survival is 1 on the whole support
     // (a point mass: every mass partial is the integral below its position,
-    // A once it has been reached, else the whole integral)
-    const float above = pm && kb >= 0 ? A[i] : C[i];
+    // Cs once it has been reached, else the whole integral)
+    const float above = pm && kb >= 0 ? Cs[i] : C[i];
     for (int q = (kb < 0 ? 0 : kb + 1); q < B; ++q) *out(1 + i, q) = above;
   }
 }
