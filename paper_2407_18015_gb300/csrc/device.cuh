@@ -515,9 +515,11 @@ __device__ __constant__ const float kGLx[4] = {0.18343464249564978f, 0.525532409
 __device__ __constant__ const float kGLw[4] = {0.36268378337836166f, 0.3137066458778869f,
                                                0.22238103445337443f, 0.10122853629037706f};
 
-// Gauss-Legendre rules on [-1, 1] with 3, 5 and 6 nodes (all nodes,
+// Gauss-Legendre rules on [-1, 1] with 2, 3, 5 and 6 nodes (all nodes,
 // ascending: the roots of P_n, weights 2 / ((1 - x^2) P_n'(x)^2)); the n-point
 // rule is exact for polynomials of degree <= 2n - 1.
+__device__ __constant__ const float kGL2x[2] = {-0.57735026918962573f, 0.57735026918962573f};
+__device__ __constant__ const float kGL2w[2] = {1.f, 1.f};
 __device__ __constant__ const float kGL3x[3] = {-0.7745966692414834f, 0.f, 0.7745966692414834f};
 __device__ __constant__ const float kGL3w[3] = {0.55555555555555569f, 0.88888888888888884f,
                                                 0.55555555555555569f};
@@ -543,10 +545,11 @@ __device__ __constant__ const float kGL16w[8] = {
     0.18945061045506864f, 0.18260341504492364f, 0.16915651939500265f, 0.14959598881657671f,
     0.12462897125553407f, 0.095158511682492605f, 0.062253523938647456f, 0.027152459411754176f};
 
-// node / weight q (ascending) of the NG-point rule, NG in {3, 5, 6, 8, 16}
+// node / weight q (ascending) of the NG-point rule, NG in {2, 3, 5, 6, 8, 16}
 template <int NG>
 __device__ __forceinline__ float gl_x(int q) {
   if constexpr (NG == 16) return q < 8 ? -kGL16x[7 - q] : kGL16x[q - 8];
+  else if constexpr (NG == 2) return kGL2x[q];
   else if constexpr (NG == 3) return kGL3x[q];
   else if constexpr (NG == 5) return kGL5x[q];
   else if constexpr (NG == 6) return kGL6x[q];
@@ -555,6 +558,7 @@ __device__ __forceinline__ float gl_x(int q) {
 template <int NG>
 __device__ __forceinline__ float gl_w(int q) {
   if constexpr (NG == 16) return q < 8 ? kGL16w[7 - q] : kGL16w[q - 8];
+  else if constexpr (NG == 2) return kGL2w[q];
   else if constexpr (NG == 3) return kGL3w[q];
   else if constexpr (NG == 5) return kGL5w[q];
   else if constexpr (NG == 6) return kGL6w[q];
@@ -570,44 +574,66 @@ __device__ __forceinline__ float epan_surv(float u) {
 
 // Gauss-Legendre rule of a piece on which J survivals (degree 3 each) and the
 // centre density (degree 2) are polynomials: the n-point rule with 2n - 1 >=
-// 2 + 3J is exact (n = 3, 5, 6, 8 for J = 1..4; 16 for the J = 5..8 of larger
-// stencils).
+// 2 + 3J is exact (n = 2, 3, 5, 6, 8 for J = 0..4; 16 for the J = 5..8 of
+// larger stencils).
 template <int J>
 struct EpanNodes {
-  static constexpr int value = J == 1 ? 3 : (J == 2 ? 5 : (J == 3 ? 6 : (J == 4 ? 8 : 16)));
+  static constexpr int value =
+      J == 0 ? 2 : (J == 1 ? 3 : (J == 2 ? 5 : (J == 3 ? 6 : (J == 4 ? 8 : 16))));
 };
 __host__ __device__ constexpr float epan_scale4(int J) { return J == 0 ? 1.f : 0.25f * epan_scale4(J - 1); }
 
-// int over a piece (middle mid, half width half) of (1 - u^2) prod_{i<J} S_i,
-// u = x iw1 and S_i = q_i^2 (3 - q_i) / 4 the survival of factor i at q_i = 1 -
-// (its argument) in [0, 2].  On the piece q_i = qm_i - qd_i xi is linear in
-// the node xi, so a node takes one multiply-add per factor for q_i, and the
-// squares and the quarters are taken once per node and piece: 4 J + 4
-// operations per node, where each factor's argument, clamp and cubic on its
-// own took 7 J + 6 (Epanechnikov saddle of 500 x 500 x 20: 41 -> 24.6 us; three
-// models of 1024 x 1024 x 20: 222 -> 211 us).  Nodes in pairs, one per half of a float2 (packed FP32
-// instructions).
+// 1 / w1 of the centre in two floats: hi the approximate reciprocal, lo its
+// residual, so that x / w1 = fma(x, hi, x lo) to one rounding.  It scales every
+// node's argument and the result, where its own rounding does not average out.
+struct EpanInv {
+  float hi, lo;
+  __device__ __forceinline__ explicit EpanInv(float w1) : hi(frcp(w1)) {
+    lo = hi * fmaf(-w1, hi, 1.f);
+  }
+  __device__ __forceinline__ float times(float x) const { return fmaf(x, hi, x * lo); }
+  __device__ __forceinline__ float2 times(float2 x) const {
+    return __ffma2_rn(x, make_float2(hi, hi), __fmul2_rn(x, make_float2(lo, lo)));
+  }
+};
+
+// int over a piece of (1 - u^2) prod_{i<J} S_i (middle mid + merr, mid rounded
+// and merr its error; half width half), u = x / w1 and S_i = q_i^2 (3 - q_i) /
+// 4 the survival of factor i at q_i = c0_i - (x - d_i) iw_i in [0, 2].  The
+// squares and the quarters are taken once per node and piece: 5 J + 7
+// operations per node, where each factor's argument, clamp and cubic on its own
+// took 7 J + 6.  Each node forms its q_i anew, and the middle and 1 / w1 are
+// taken to two floats: with q_i = qm_i - qd_i xi and single floats (4 J + 4
+// operations) their roundings are common to all nodes of a piece, and the mean
+// error against 64 bits was 10 to 25 % larger than that of the form with one
+// factor at a time; now the two are equal.  Nodes in pairs, one per half of a
+// float2 (packed FP32 instructions).  1024 x 1024 vertices from parameters:
+// minimum and maximum 50 us, saddle 77 (one factor at a time 56 and 130, single
+// floats 44 and 62); three models of 1024 x 1024 x 20 220 us (224, 218).
+// A factor that starts at the range's end enters pieces of zero width alone,
+// where nothing bounds q: they are 0.
 // NG: the rule, if fewer nodes do (the product is known to have a lower
 // degree).
 template <int J, int NG = EpanNodes<J>::value>
-__device__ __forceinline__ float epan_piece(float mid, float half, float iw1, const float *qm,
-                                            const float *qd) {
-  const float um = mid * iw1, ud = half * iw1;
-  if constexpr (J == 0) {
-    // the mean of 1 - u^2
-    return 2.f * half * fmaf(-um, um, fmaf(-ud * (1.f / 3.f), ud, 1.f));
-  } else {
-    const float2 one2 = make_float2(1.f, 1.f), three2 = make_float2(3.f, 3.f);
-    float2 s2 = make_float2(0.f, 0.f);
+__device__ __forceinline__ float epan_piece(float mid, float merr, float half, EpanInv iw1,
+                                            const float *d, const float *iw, const float *c0) {
+  const float2 one2 = make_float2(1.f, 1.f), three2 = make_float2(3.f, 3.f);
+  float2 s2 = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int n = 0; n + 1 < NG; n += 2) {
-      const float2 xi = make_float2(gl_x<NG>(n), gl_x<NG>(n + 1));
-      const float2 u = __ffma2_rn(make_float2(ud, ud), xi, make_float2(um, um));
-      const float2 g = __ffma2_rn(make_float2(-u.x, -u.y), u, one2);
+  for (int n = 0; n + 1 < NG; n += 2) {
+    const float2 xi = make_float2(gl_x<NG>(n), gl_x<NG>(n + 1));
+    const float2 x = __fadd2_rn(__ffma2_rn(make_float2(half, half), xi, make_float2(merr, merr)),
+                                make_float2(mid, mid));
+    const float2 u = iw1.times(x);
+    const float2 g = __ffma2_rn(make_float2(-u.x, -u.y), u, one2);
+    if constexpr (J == 0) {
+      s2 = __ffma2_rn(make_float2(gl_w<NG>(n), gl_w<NG>(n + 1)), g, s2);
+    } else {
       float2 Q = one2, T = one2;
 #pragma unroll
       for (int i = 0; i < J; ++i) {
-        const float2 q = __ffma2_rn(make_float2(-qd[i], -qd[i]), xi, make_float2(qm[i], qm[i]));
+        const float2 e = __fadd2_rn(make_float2(d[i], d[i]), make_float2(-x.x, -x.y));
+        const float2 q = __ffma2_rn(e, make_float2(iw[i], iw[i]), make_float2(c0[i], c0[i]));
         const float2 t = __fadd2_rn(three2, make_float2(-q.x, -q.y));
         Q = i == 0 ? q : __fmul2_rn(Q, q);
         T = i == 0 ? t : __fmul2_rn(T, t);
@@ -615,39 +641,35 @@ __device__ __forceinline__ float epan_piece(float mid, float half, float iw1, co
       const float2 f = __fmul2_rn(__fmul2_rn(Q, Q), __fmul2_rn(T, g));
       s2 = __ffma2_rn(make_float2(gl_w<NG>(n), gl_w<NG>(n + 1)), f, s2);
     }
-    float s = s2.x + s2.y;
-    if constexpr (NG & 1) {
-      constexpr int n = NG - 1;
-      const float u = fmaf(ud, gl_x<NG>(n), um);
-      float Q = 1.f, T = fmaf(-u, u, 1.f);
-#pragma unroll
-      for (int i = 0; i < J; ++i) {
-        const float q = fmaf(-qd[i], gl_x<NG>(n), qm[i]);
-        Q *= q;
-        T *= 3.f - q;
-      }
-      s = fmaf(gl_w<NG>(n) * (Q * Q), T, s);
-    }
-    return s * (half * epan_scale4(J));
   }
+  float s = s2.x + s2.y;
+  if constexpr (NG & 1) {
+    constexpr int n = NG - 1;
+    const float x = fmaf(half, gl_x<NG>(n), merr) + mid, u = iw1.times(x);
+    float Q = 1.f, T = fmaf(-u, u, 1.f);
+#pragma unroll
+    for (int i = 0; i < J; ++i) {
+      const float q = fmaf(d[i] - x, iw[i], c0[i]);
+      Q *= q;
+      T *= 3.f - q;
+    }
+    s = fmaf(gl_w<NG>(n) * (Q * Q), T, s);
+  }
+  return half > 0.f ? s * (half * epan_scale4(J)) : 0.f;
 }
 
 // Pieces J.. of epan_side: on [x[J], x[J+1]] the sorted factors 0..J-1 have
 // started.  A started factor's argument lies in [-1, 1] there (the piece
 // begins after the factor's start, and R is at most every present
-// neighbour's end); a factor that starts at R enters pieces of zero width
-// alone, where q is held at 2 (its survival at 1) so that nothing overflows.
+// neighbour's end).
 template <int J, int K, int NP>
-__device__ __forceinline__ void epan_pieces(const float *x, const float (*pay)[NP], float iw1,
+__device__ __forceinline__ void epan_pieces(const float *x, const float (*pay)[NP], EpanInv iw1,
                                             Kahan &acc) {
   const float half = 0.5f * (x[J + 1] - x[J]), mid = 0.5f * (x[J] + x[J + 1]);
-  float qm[J > 0 ? J : 1], qd[J > 0 ? J : 1];
+  float c0[J > 0 ? J : 1];
 #pragma unroll
-  for (int i = 0; i < J; ++i) {
-    qm[i] = fminf(fmaf(-(mid - pay[0][i]), pay[1][i], 1.f), 2.f);
-    qd[i] = half * pay[1][i];
-  }
-  acc.add(epan_piece<J>(mid, half, iw1, qm, qd));
+  for (int i = 0; i < J; ++i) c0[i] = 1.f;
+  acc.add(epan_piece<J>(mid, (x[J] - mid) + half, half, iw1, pay[0], pay[1], c0));
   if constexpr (J < K) epan_pieces<J + 1, K, NP>(x, pay, iw1, acc);
 }
 
@@ -668,10 +690,10 @@ __device__ __forceinline__ float epan_side(float w1, float L, float R, float al[
   }
   sort4<2>(t, pay);
   const float x[6] = {L, t[0], t[1], t[2], t[3], R};
-  const float iw1 = frcp(w1);
+  const EpanInv iw1(w1);
   Kahan acc;
   epan_pieces<0, 4, 4>(x, pay, iw1, acc);
-  return not_negative(0.75f * iw1 * acc.get());
+  return not_negative(iw1.times(0.75f * acc.get()));
 }
 
 struct EpanParams {
@@ -713,7 +735,7 @@ __device__ __forceinline__ void epan_vertex(EpanParams c, const EpanParams *nb,
           al[i] = kFar; d[i] = kFar; iw[i] = 0.f;
           R = fminf(R, dn);
         } else {
-          al[i] = dn - wn; d[i] = dn; iw[i] = rcp_held(frcp(wn));
+          al[i] = dn - wn; d[i] = dn; iw[i] = frcp(wn);
           R = fminf(R, dn + wn);
         }
       } else {
@@ -733,7 +755,7 @@ __device__ __forceinline__ void epan_vertex(EpanParams c, const EpanParams *nb,
           al[i] = kFar; d[i] = kFar; iw[i] = 0.f;
           R = fminf(R, dn);
         } else {
-          al[i] = dn - wn; d[i] = dn; iw[i] = rcp_held(frcp(wn));
+          al[i] = dn - wn; d[i] = dn; iw[i] = frcp(wn);
           R = fminf(R, dn + wn);
         }
       } else {
@@ -969,21 +991,20 @@ __device__ __forceinline__ float uniform_mixed(UniParams c, const UniParams *nb,
 // up to its start and a polynomial beyond, so at most two factors are
 // polynomials before the first breakpoint, three after one of them, four after
 // two, three and two after the next: rules of 5, 6, 8, 6 and 5 points are exact
-// (30 nodes, 40 with eight on every piece: 500 x 500 x 20 24.6 -> 22.5 us).
+// (30 nodes, 40 with eight on every piece).
 template <int J>
 __device__ __forceinline__ void epan_mixed_pieces(const float *x, const float *d, const float *iw,
-                                                  float iw1, Kahan &acc) {
+                                                  EpanInv iw1, Kahan &acc) {
   constexpr int NG = J == 2 ? 8 : ((J & 1) ? 6 : 5);
   const float half = 0.5f * (x[J + 1] - x[J]), mid = 0.5f * (x[J] + x[J + 1]);
-  float qm[4], qd[4];
+  float iwp[4], c0[4];  // the constant 1: q = 2
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const float q = fmaf(-(mid - d[i]), iw[i], 1.f);
-    const bool one = iw[i] == 0.f || q >= 2.f;
-    qm[i] = one ? 2.f : q;
-    qd[i] = one ? 0.f : half * iw[i];
+    const bool one = iw[i] == 0.f || fmaf(d[i] - mid, iw[i], 1.f) >= 2.f;
+    iwp[i] = one ? 0.f : iw[i];
+    c0[i] = one ? 2.f : 1.f;
   }
-  acc.add(epan_piece<4, NG>(mid, half, iw1, qm, qd));
+  acc.add(epan_piece<4, NG>(mid, (x[J] - mid) + half, half, iw1, d, iwp, c0));
   if constexpr (J < 4) epan_mixed_pieces<J + 1>(x, d, iw, iw1, acc);
 }
 
@@ -1015,10 +1036,10 @@ __device__ __forceinline__ float epan_mixed(EpanParams c, const EpanParams *nb, 
     const float dn = nb[i].m - c.m, wn = nb[i].w;
     if (sg[i] > 0) {
       R = fminf(R, dn + wn);
-      if (wn > 0.f) { bp[i] = dn - wn; d[i] = dn; iw[i] = rcp_held(frcp(wn)); }
+      if (wn > 0.f) { bp[i] = dn - wn; d[i] = dn; iw[i] = frcp(wn); }
     } else {
       L = fmaxf(L, dn - wn);
-      if (wn > 0.f) { bp[i] = dn + wn; d[i] = dn; iw[i] = -rcp_held(frcp(wn)); }
+      if (wn > 0.f) { bp[i] = dn + wn; d[i] = dn; iw[i] = -frcp(wn); }
     }
   }
   if (!(R > L)) return 0.f;
@@ -1028,10 +1049,10 @@ __device__ __forceinline__ float epan_mixed(EpanParams c, const EpanParams *nb, 
   float none[1][4];
   sort4<0>(t, none);
   const float x[6] = {L, t[0], t[1], t[2], t[3], R};
-  const float iw1 = frcp(w1);
+  const EpanInv iw1(w1);
   Kahan acc;
   epan_mixed_pieces<0>(x, d, iw, iw1, acc);
-  return not_negative(0.75f * iw1 * acc.get());
+  return not_negative(iw1.times(0.75f * acc.get()));
 }
 
 // saddle signs of the four slots (e, n, w, s) for t1, or all zero when the

@@ -202,7 +202,7 @@ __device__ __forceinline__ void uniform_vertex_k(UniParams c, const UniParams *n
 
 // ---------------------------------------------------------------------------
 // Epanechnikov: with K neighbours the integrand has degree <= 2 + 3K = 26 on
-// a piece; each piece takes the smallest rule of {3, 5, 6, 8, 16} nodes that
+// a piece; each piece takes the smallest rule of {2, 3, 5, 6, 8, 16} nodes that
 // is exact for its degree (EpanNodes; the 16-point rule: to degree 31)
 
 // epan_side with K factors (same frame and arguments)
@@ -223,10 +223,10 @@ __device__ __forceinline__ float epan_side_k(float w1, float L, float R, const f
 #pragma unroll
   for (int i = 0; i < K; ++i) x[i + 1] = t[i];
   x[K + 1] = R;
-  const float iw1 = frcp(w1);
+  const EpanInv iw1(w1);
   Kahan acc;
   epan_pieces<0, K, kMaxK>(x, pay, iw1, acc);
-  return not_negative(0.75f * iw1 * acc.get());
+  return not_negative(iw1.times(0.75f * acc.get()));
 }
 
 template <int K>
@@ -268,7 +268,7 @@ __device__ __forceinline__ void epan_vertex_k(EpanParams c, const EpanParams *nb
       if (wn == 0.f) {  // point mass: survival 1 below it, and it caps R
         R = fminf(R, dn);
       } else {
-        al[i] = dn - wn; d[i] = dn; iw[i] = rcp_held(frcp(wn));
+        al[i] = dn - wn; d[i] = dn; iw[i] = frcp(wn);
         R = fminf(R, dn + wn);
       }
     }
