@@ -159,7 +159,7 @@ int ucp_launch_fused3(ucp_ctx *ctx, const float *ens, int N, int H, int W,
     F.out_max[sl] = (cptypes & 2u) ? out_max[m] : nullptr;
     F.status[sl] = status ? status[m] : nullptr;
   }
-  return ucp_set_error(ctx, launch_closed3(F, stream, launched));
+  return ucp_set_error(ctx, launch_closed3(F, ctx->sm_count, stream, launched));
 }
 
 extern "C" {

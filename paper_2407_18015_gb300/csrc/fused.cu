@@ -28,7 +28,6 @@ namespace {
 
 constexpr int kTY3 = 8, kHALO3 = (kTY3 + 2) * 34, kRS3 = hist_r4_stride(kHALO3);
 constexpr int kOcc3 = 3;  // resident CTAs per SM
-constexpr int kSplitCtas = 152;  // one CTA per SM
 
 // Shared memory of a fused tile, in floats: the member box, whose room the
 // histogram's per-bin rows take after the last read of the box; the
@@ -378,7 +377,7 @@ __global__ void __launch_bounds__(NTHREADS, kOcc3)
 
 }  // namespace
 
-cudaError_t launch_closed3(const Field3 &F, cudaStream_t s, bool *launched) {
+cudaError_t launch_closed3(const Field3 &F, int sm_count, cudaStream_t s, bool *launched) {
   *launched = false;
   const Field &f = F.f;
   if (f.B < 1 || f.B > 8 || f.N < 1 || f.N > 65535) return cudaSuccess;
@@ -435,13 +434,16 @@ cudaError_t launch_closed3(const Field3 &F, cudaStream_t s, bool *launched) {
   Field3 G = F;
   G.f.tma_nc = nc;
   const size_t smem = std::max((size_t)nc * per_member, rows_b) + fixed_b;
-  // A grid whose tiles leave SMs empty even three times over (up to 50 tiles
-  // of 8 x 32: a 64 x 64 field has 16) takes three CTAs per tile, one per
-  // model: each then waits for one model's chain of stages and not for the
-  // sum of the three, and staging a tile three times costs nothing there
-  // (64 x 64 x 20: 13.1 -> 10.9 us a
-  // launch, launch included; 128 x 128 x 20, 64 tiles: 13.4 -> 15.1)
-  const bool split = tiles * 3 <= kSplitCtas;
+  // A grid whose tiles leave SMs empty even three times over (152 SMs: up to 50
+  // tiles of 8 x 32; a 64 x 64 field has 16) takes three CTAs per tile, one per
+  // model: each then waits for one model's chain of stages and not for the sum
+  // of the three, and staging a tile three times costs nothing there.  One
+  // against three CTAs per tile, 20 members, launch included: 16 tiles 13.6 and
+  // 11.5 us, 24 to 50 tiles 13.6 and 11.5 to 11.7 (5 members 12.2 to 12.5 and
+  // 10.1 to 10.5, 60 members 18.8 and 16.7 to 17.2).  Beyond one CTA per SM the
+  // gain shrinks (52 tiles 12.3, 56 tiles 12.8) and is lost at 60 (13.7 and
+  // 15.6).
+  const bool split = tiles * 3 <= sm_count;
   auto k = split ? (tma ? tile3_kernel<false, true> : tile3_kernel<true, true>)
                  : (tma ? tile3_kernel<false, false> : tile3_kernel<true, false>);
   k<<<dim3((unsigned)tiles, split ? 3u : 1u), NTHREADS, smem, s>>>(G, tiles_x, map);

@@ -48,7 +48,7 @@ struct Field3 {
 };
 // Launches the fused kernel when it applies (any member alignment, at most 8
 // bins and 65535 members); *launched tells whether it did.
-cudaError_t launch_closed3(const Field3 &f, cudaStream_t s, bool *launched);
+cudaError_t launch_closed3(const Field3 &f, int sm_count, cudaStream_t s, bool *launched);
 // cuTensorMapEncodeTiled from the driver (nullptr if unavailable)
 void *tensor_map_encoder_fn();
 // TMA staging plan of one field for the single-field tile kernels' layout
