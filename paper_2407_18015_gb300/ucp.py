@@ -145,8 +145,11 @@ def _stream(stream=None, device=None):
     current device) without building a torch.cuda.Stream for it."""
     if stream is not None:
         return stream.cuda_stream
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:  # not part of torch's public interface
+        return torch.cuda.current_stream(device).cuda_stream
     idx = device.index if device is not None else None
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device() if idx is None else idx)
+    return raw(torch.cuda.current_device() if idx is None else idx)
 
 
 def make_desc(model="uniform", bins=8, epan_width_scale=0.0, mc_samples=10000, seed=0x5EED,
