@@ -4,7 +4,7 @@
 // compares against (Sec. "Comparison of Parametric Vs. Nonparametric
 // Models", multivariate Gaussian with Monte Carlo sampling).
 //
-// One warp per vertex.  Lanes split the samples, two per turn; each sample
+// One warp per vertex.  Lanes split the samples, one or two per turn; each sample
 // draws two Philox4x32-10 blocks (counter (s, vertex, field, j), key = seed),
 // maps the words to uniforms ((r >> 9) + 0.5) 2^-23 (exact in binary32, inside
 // (0, 1)), and Box-Muller gives six normals, five of which are used.  The
@@ -32,35 +32,60 @@ __device__ __forceinline__ void philox_pair(uint32_t s, uint32_t v, uint32_t fie
   }
 }
 
-// The words of two samples (one per half) as 1 + m 2^-23, m their upper 23
-// bits: the uniforms are these minus 1 - 2^-24, exactly.
-__device__ __forceinline__ float2 word_pair(uint32_t r0, uint32_t r1) {
-  return make_float2(__uint_as_float((r0 >> 9) + 0x3f800000u),
-                     __uint_as_float((r1 >> 9) + 0x3f800000u));
+// Arithmetic of the samples of one lane and turn, every operation rounded
+// once: two (PAIR, one per half of a float2) or one, to the same bits.
+template <bool PAIR>
+struct McOps {
+  static constexpr int n = 2;
+  using V = float2;
+  static __device__ __forceinline__ V add(V a, V b) { return __fadd2_rn(a, b); }
+  static __device__ __forceinline__ V mul(V a, V b) { return __fmul2_rn(a, b); }
+  static __device__ __forceinline__ V fma(V a, V b, V c) { return __ffma2_rn(a, b, c); }
+  static __device__ __forceinline__ V all(float a) { return make_float2(a, a); }
+  static __device__ __forceinline__ float &at(V &a, int h) { return h == 0 ? a.x : a.y; }
+};
+template <>
+struct McOps<false> {
+  static constexpr int n = 1;
+  using V = float;
+  static __device__ __forceinline__ V add(V a, V b) { return __fadd_rn(a, b); }
+  static __device__ __forceinline__ V mul(V a, V b) { return __fmul_rn(a, b); }
+  static __device__ __forceinline__ V fma(V a, V b, V c) { return __fmaf_rn(a, b, c); }
+  static __device__ __forceinline__ V all(float a) { return a; }
+  static __device__ __forceinline__ float &at(V &a, int) { return a; }
+};
+
+// A Philox word as 1 + m 2^-23, m its upper 23 bits: the uniform is this minus
+// 1 - 2^-24, exactly.
+__device__ __forceinline__ float word_float(uint32_t r) {
+  return __uint_as_float((r >> 9) + 0x3f800000u);
 }
 
-// Box-Muller of two samples (one per half of the float2s), wa and wb their
-// words as word_pair gives them: radius sqrt(-2 ln ua), angle 2 pi ub.  The
-// angle is taken as pi + t with t = 2 pi (ub - 1/2) in [-pi, pi), where the
+// Box-Muller of a turn's samples, wa and wb their words as word_float gives
+// them: radius sqrt(-2 ln ua), angle 2 pi ub.  The angle is taken as pi + t with t = 2 pi (ub - 1/2) in [-pi, pi), where the
 // hardware sine and cosine are accurate to ~4e-7 absolute: cos(2 pi ub) = -cos
 // t, sin(2 pi ub) = -sin t.  ub - 1/2 = (wb - 3/2) + 2^-24 exactly, so one
 // multiply-add gives t with the rounding of the product.  The logarithm keeps
 // full accuracy (its error is not bounded relative to the radius near ub ->
 // 1).  Z1: also the second normal.
-template <bool Z1>
-__device__ __forceinline__ void box_muller2(float2 wa, float2 wb, float2 &z0, float2 &z1) {
-  const float c1 = -(1.f - 0x1p-24f), twopi = 6.283185307179586f;
-  const float2 ua = __fadd2_rn(wa, make_float2(c1, c1));
-  const float2 v = __fmul2_rn(make_float2(-2.f, -2.f), make_float2(logf(ua.x), logf(ua.y)));
-  const float2 rad = __fmul2_rn(v, make_float2(rsqrtf(v.x), rsqrtf(v.y)));
-  const float2 t = __ffma2_rn(__fadd2_rn(wb, make_float2(-1.5f, -1.5f)), make_float2(twopi, twopi),
-                              make_float2(twopi * 0x1p-24f, twopi * 0x1p-24f));
-  float2 sn, cs;
-  __sincosf(t.x, &sn.x, &cs.x);
-  __sincosf(t.y, &sn.y, &cs.y);
-  const float2 nr = make_float2(-rad.x, -rad.y);
-  z0 = __fmul2_rn(nr, cs);
-  if constexpr (Z1) z1 = __fmul2_rn(nr, sn);
+template <typename O, bool Z1, typename V>
+__device__ __forceinline__ void box_muller(V wa, V wb, V &z0, V &z1) {
+  const float twopi = 6.283185307179586f;
+  V ua = O::add(wa, O::all(-(1.f - 0x1p-24f))), ln, rs, sn, cs;
+#pragma unroll
+  for (int h = 0; h < O::n; ++h) O::at(ln, h) = logf(O::at(ua, h));
+  V v = O::mul(O::all(-2.f), ln);
+#pragma unroll
+  for (int h = 0; h < O::n; ++h) O::at(rs, h) = rsqrtf(O::at(v, h));
+  V rad = O::mul(v, rs);
+  V t = O::fma(O::add(wb, O::all(-1.5f)), O::all(twopi), O::all(twopi * 0x1p-24f));
+#pragma unroll
+  for (int h = 0; h < O::n; ++h) {
+    __sincosf(O::at(t, h), &O::at(sn, h), &O::at(cs, h));
+    O::at(rad, h) = -O::at(rad, h);
+  }
+  z0 = O::mul(rad, cs);
+  if constexpr (Z1) z1 = O::mul(rad, sn);
 }
 
 // Slots of the variables: 0 = v, 1..4 = e, n, w, s.  Returns the number of
@@ -172,63 +197,85 @@ __global__ void __launch_bounds__(256) mvn_fit_kernel(Field f) {
 // (SADDLE) the saddle in h0.  D, M: y_n = D[n] + sum_b M[n][b] z_b of the nv
 // present variables; FULL: nv = 5 (no test per neighbour).  Bound by
 // instruction issue, about 240 a sample, 35 of them 64-bit Philox products
-// (four FP32-pipe cycles each): two samples per turn, so that every FP32
+// (four FP32-pipe cycles each): with two samples per turn (PAIR) every FP32
 // operation but the logarithms and the special functions is a packed one (the
 // same roundings as one by one): 512 x 512 x 40, 10^4 samples 22.2 ->
 // 19.4 ms.
-template <bool SADDLE, bool FULL>
+template <bool SADDLE, bool FULL, bool PAIR>
 __device__ __forceinline__ void mc_count(int S, int lane, uint32_t vid, uint32_t field,
                                          const PhiloxKeys &K, const float *D,
                                          const float (&M)[5][5], int nv, const float *ssg,
                                          bool has_saddle, unsigned &h0, unsigned &h1) {
-  auto two = [&](uint32_t s0, uint32_t s1, bool second) {
-    uint4 a0, a1, b0, b1;
-    philox_pair(s0, vid, field, K, a0, a1);
-    philox_pair(s1, vid, field, K, b0, b1);
-    float2 z[6];
-    box_muller2<true>(word_pair(a0.x, b0.x), word_pair(a0.y, b0.y), z[0], z[1]);
-    box_muller2<true>(word_pair(a0.z, b0.z), word_pair(a0.w, b0.w), z[2], z[3]);
-    box_muller2<false>(word_pair(a1.x, b1.x), word_pair(a1.y, b1.y), z[4], z[5]);
+  using O = McOps<PAIR>;
+  using V = typename O::V;
+  // samples s and, in a pair, s + 32 (computed, but only counted if `second`)
+  auto turn = [&](uint32_t s, bool second) {
+    V w[2][4];
+#pragma unroll
+    for (int h = 0; h < O::n; ++h) {
+      uint4 r0, r1;
+      philox_pair(s + 32u * h, vid, field, K, r0, r1);
+      O::at(w[0][0], h) = word_float(r0.x);
+      O::at(w[0][1], h) = word_float(r0.y);
+      O::at(w[0][2], h) = word_float(r0.z);
+      O::at(w[0][3], h) = word_float(r0.w);
+      O::at(w[1][0], h) = word_float(r1.x);
+      O::at(w[1][1], h) = word_float(r1.y);
+    }
+    V z[6];
+    box_muller<O, true>(w[0][0], w[0][1], z[0], z[1]);
+    box_muller<O, true>(w[0][2], w[0][3], z[2], z[3]);
+    box_muller<O, false>(w[1][0], w[1][1], z[4], z[5]);
     // x_v below every neighbour: the largest y_n = x_v - x_n is < 0;
     // above every one: the smallest is > 0
-    float2 ymax = make_float2(-kFar, -kFar), ymin = make_float2(kFar, kFar);
-    bool t1x = has_saddle, t2x = has_saddle, t1y = has_saddle, t2y = has_saddle;
+    float ymax[O::n], ymin[O::n];
+    bool t1[O::n], t2[O::n];
+#pragma unroll
+    for (int h = 0; h < O::n; ++h) {
+      ymax[h] = -kFar;
+      ymin[h] = kFar;
+      t1[h] = t2[h] = has_saddle;
+    }
 #pragma unroll
     for (int n = 1; n < 5; ++n) {
       if (FULL || n < nv) {
-        float2 yv = make_float2(D[n], D[n]);
+        V yv = O::all(D[n]);
 #pragma unroll
-        for (int b = 0; b <= n; ++b) yv = __ffma2_rn(make_float2(M[n][b], M[n][b]), z[b], yv);
-        if constexpr (SADDLE) {
-          // t1 wants x_v < x_n where the sign is +1
-          const float sx = ssg[n] * yv.x, sy = ssg[n] * yv.y;
-          t1x &= sx < 0.f;
-          t2x &= sx > 0.f;
-          t1y &= sy < 0.f;
-          t2y &= sy > 0.f;
-        } else {
-          ymax = make_float2(fmaxf(ymax.x, yv.x), fmaxf(ymax.y, yv.y));
-          ymin = make_float2(fminf(ymin.x, yv.x), fminf(ymin.y, yv.y));
+        for (int b = 0; b <= n; ++b) yv = O::fma(O::all(M[n][b]), z[b], yv);
+#pragma unroll
+        for (int h = 0; h < O::n; ++h) {
+          const float y = O::at(yv, h);
+          if constexpr (SADDLE) {
+            // t1 wants x_v < x_n where the sign is +1
+            const float sy = ssg[n] * y;
+            t1[h] &= sy < 0.f;
+            t2[h] &= sy > 0.f;
+          } else {
+            ymax[h] = fmaxf(ymax[h], y);
+            ymin[h] = fminf(ymin[h], y);
+          }
         }
       }
     }
-    if constexpr (SADDLE) {
-      h0 += (t1x || t2x) ? 1u : 0u;
-      h0 += (second && (t1y || t2y)) ? 1u : 0u;
-    } else {
-      h0 += ymax.x < 0.f ? 1u : 0u;
-      h1 += ymin.x > 0.f ? 1u : 0u;
-      h0 += (second && ymax.y < 0.f) ? 1u : 0u;
-      h1 += (second && ymin.y > 0.f) ? 1u : 0u;
+#pragma unroll
+    for (int h = 0; h < O::n; ++h) {
+      const bool count = h == 0 || second;
+      if constexpr (SADDLE) {
+        h0 += (count && (t1[h] || t2[h])) ? 1u : 0u;
+      } else {
+        h0 += (count && ymax[h] < 0.f) ? 1u : 0u;
+        h1 += (count && ymin[h] > 0.f) ? 1u : 0u;
+      }
     }
   };
-  const uint32_t whole = (uint32_t)S & ~63u;
-  for (uint32_t s = 0; s < whole; s += 64) two(s + lane, s + 32 + lane, true);
+  constexpr uint32_t step = 32 * O::n;
+  const uint32_t whole = (uint32_t)S / step * step;
+  for (uint32_t s = 0; s < whole; s += step) turn(s + lane, true);
   const uint32_t s = whole + lane;
-  if (s < (uint32_t)S) two(s, s + 32, s + 32 < (uint32_t)S);
+  if (s < (uint32_t)S) turn(s, s + 32 < (uint32_t)S);
 }
 
-template <bool FROM_MEMBERS, bool SADDLE>
+template <bool FROM_MEMBERS, bool SADDLE, bool PAIR>
 __global__ void __launch_bounds__(256) mvn_mc_kernel(Field f, int S, uint32_t k0, uint32_t k1,
                                                      uint32_t field) {
   const int lane = threadIdx.x & 31;
@@ -373,9 +420,9 @@ __global__ void __launch_bounds__(256) mvn_mc_kernel(Field f, int S, uint32_t k0
         unsigned h0 = 0, h1 = 0;
         const PhiloxKeys K(k0, k1);
         if (nv == 5)
-          mc_count<SADDLE, true>(S, lane, (uint32_t)v, field, K, D, M, nv, ssg, has_saddle, h0, h1);
+          mc_count<SADDLE, true, PAIR>(S, lane, (uint32_t)v, field, K, D, M, nv, ssg, has_saddle, h0, h1);
         else
-          mc_count<SADDLE, false>(S, lane, (uint32_t)v, field, K, D, M, nv, ssg, has_saddle, h0, h1);
+          mc_count<SADDLE, false, PAIR>(S, lane, (uint32_t)v, field, K, D, M, nv, ssg, has_saddle, h0, h1);
         const unsigned cmin = __reduce_add_sync(0xffffffffu, h0), csad = cmin;
         const unsigned cmax = __reduce_add_sync(0xffffffffu, h1);
         pmin = zero_mm ? 0.f : (float)cmin / (float)S;
@@ -408,6 +455,24 @@ cudaError_t launch_mvn_fit(const Field &f, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// Two samples per turn take 80 to 93 registers a thread (one: 64) and work on
+// 64 samples at a time: few samples go one per turn, for the occupancy of the
+// part before the samples.  512 x 512 x 20, one and two per turn: minimum and
+// maximum 376 and 459 us at 32 samples, 546 and 559 at 128, 737 and 763 at 224,
+// 800 and 769 at 256, 2353 and 2192 at 1000; saddle 401 and 568 at 32, 820 and
+// 890 at 256, 1337 and 1351 at 512, 1863 and 1811 at 768.
+constexpr int kMcPairs = 225, kMcPairsSaddle = 513;
+
+template <bool SADDLE>
+static cudaError_t launch_mc(const Field &f, bool from_members, int samples, uint32_t k0,
+                             uint32_t k1, uint32_t field_id, int blocks, cudaStream_t s) {
+  const bool pair = samples >= (SADDLE ? kMcPairsSaddle : kMcPairs);
+  auto k = from_members ? (pair ? mvn_mc_kernel<true, SADDLE, true> : mvn_mc_kernel<true, SADDLE, false>)
+                        : (pair ? mvn_mc_kernel<false, SADDLE, true> : mvn_mc_kernel<false, SADDLE, false>);
+  k<<<blocks, 256, 0, s>>>(f, samples, k0, k1, field_id);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_mvn_mc(const Field &f, bool from_members, int samples, uint64_t seed,
                           uint32_t field_id, cudaStream_t s) {
   // one warp per vertex, 8 warps per CTA, grid-stride over vertices
@@ -419,20 +484,10 @@ cudaError_t launch_mvn_mc(const Field &f, bool from_members, int samples, uint64
   // minimum / maximum and the saddle are separate instances, so that
   // neither pays for the other's tests in the sample loop
   cudaError_t e = cudaSuccess;
-  if (f.cptypes & (kMin | kMax)) {
-    if (from_members)
-      mvn_mc_kernel<true, false><<<(int)b, 256, 0, s>>>(f, samples, k0, k1, field_id);
-    else
-      mvn_mc_kernel<false, false><<<(int)b, 256, 0, s>>>(f, samples, k0, k1, field_id);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess && (f.cptypes & kSaddle)) {
-    if (from_members)
-      mvn_mc_kernel<true, true><<<(int)b, 256, 0, s>>>(f, samples, k0, k1, field_id);
-    else
-      mvn_mc_kernel<false, true><<<(int)b, 256, 0, s>>>(f, samples, k0, k1, field_id);
-    e = cudaGetLastError();
-  }
+  if (f.cptypes & (kMin | kMax))
+    e = launch_mc<false>(f, from_members, samples, k0, k1, field_id, (int)b, s);
+  if (e == cudaSuccess && (f.cptypes & kSaddle))
+    e = launch_mc<true>(f, from_members, samples, k0, k1, field_id, (int)b, s);
   return e;
 }
 
