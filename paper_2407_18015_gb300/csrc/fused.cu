@@ -152,6 +152,7 @@ __device__ __forceinline__ bool stage3(const Field &f, float *smh, float *sme, f
     const int l = lv[p];
     smh[l] = nf[p] ? qnan() : mn[p];
     smh[HALO + l] = nf[p] ? qnan() : mx[p];
+    if (!epan) continue;
     float m, w;
     if (mn[p] == mx[p]) {
       m = mn[p];
@@ -356,7 +357,8 @@ __global__ void __launch_bounds__(NTHREADS, kOcc3)
   float *sme = smh + htile3_floats();
   uint64_t *bar = reinterpret_cast<uint64_t *>(sme + ((etile3_floats() + 1) & ~1LL));
   float4 *R4 = reinterpret_cast<float4 *>(smem);
-  const int only = SPLIT ? (int)blockIdx.y : -1;  // one model per row of CTAs
+  // one model per row of CTAs, the histogram (the longest) first
+  const int only = SPLIT ? 2 - (int)blockIdx.y : -1;
   const bool ok = stage3<ASYNC, SPLIT>(f, smh, sme, smem, bar, &tmap, ty0, tx0, R4, only);
   __syncthreads();
   if (!ok) {  // a bounded wait gave up: NaN and the timeout flag, every model
@@ -438,11 +440,11 @@ cudaError_t launch_closed3(const Field3 &F, int sm_count, cudaStream_t s, bool *
   // tiles of 8 x 32; a 64 x 64 field has 16) takes three CTAs per tile, one per
   // model: each then waits for one model's chain of stages and not for the sum
   // of the three, and staging a tile three times costs nothing there.  One
-  // against three CTAs per tile, 20 members, launch included: 16 tiles 13.6 and
-  // 11.5 us, 24 to 50 tiles 13.6 and 11.5 to 11.7 (5 members 12.2 to 12.5 and
-  // 10.1 to 10.5, 60 members 18.8 and 16.7 to 17.2).  Beyond one CTA per SM the
-  // gain shrinks (52 tiles 12.3, 56 tiles 12.8) and is lost at 60 (13.7 and
-  // 15.6).
+  // against three CTAs per tile, launches included: 20 members 13.6 and 10.8 us
+  // at 16 tiles, 13.6 and 10.9 at 50; 5 members 12.5 and 9.3, 12.5 and 9.7; 60
+  // members 18.8 and 15.9, 18.8 and 16.2.  Beyond one CTA per SM the gain shrinks
+  // and is lost at 60 tiles (20 members, with 0.7 us more for three: 52 tiles
+  // 12.3, 56 tiles 12.8, 60 tiles 15.6).
   const bool split = tiles * 3 <= sm_count;
   auto k = split ? (tma ? tile3_kernel<false, true> : tile3_kernel<true, true>)
                  : (tma ? tile3_kernel<false, false> : tile3_kernel<true, false>);
