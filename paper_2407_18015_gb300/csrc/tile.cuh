@@ -789,7 +789,7 @@ __device__ __forceinline__ bool stage_members_tma(const Field &f, float *sm, flo
   // that hold each (member, row) segment: the element of column c (x =
   // tx0 - 4 + c) then lands at c + d, d = (its address / 4) mod 4, at most
   // 3, so the columns the staged vertices read (3 .. 36) stay inside the
-  // 40-float row.  Five threads share a segment, two blocks each; only the
+  // 40-float row (box_copy_async: a thread per block of a row).  Only the
   // blocks that hold a column a staged in-grid vertex reads are copied, so
   // every block read holds an element of the members (no read leaves the
   // allocation).  d = (eb + m pl + gy w4) mod 4 for member m and row gy (eb
