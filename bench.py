@@ -193,13 +193,13 @@ ADJ_EPAN_FLOPS_PER_VERTEX = 2 * EPAN_FLOPS_PER_VERTEX_TYPE
 # three-model kernel) and of each model's own kernel, from the ncu captures
 # summarised in profiles/; None once a kernel has changed since its counters
 # were taken
-TRAFFIC_BYTES = {"fused": 93997312, "uniform": 87995392, "epanechnikov": 84948480,
-                 "histogram": 85448448, "hist_adjoint_16": 655649280}
+TRAFFIC_BYTES = {"fused": 93955072, "uniform": 88120576, "epanechnikov": 85557248,
+                 "histogram": 85341440, "hist_adjoint_16": 655121920}
 # warp instructions per launch of the same kernels (ncu smsp__inst_executed.sum,
 # profiles/instructions_bench_headline_1024x1024x20.md): the issue-rate
 # fraction reported beside the FP32 / HBM one; None once a kernel changed
-ISSUE_WARP_INSTR = {"fused": 184748713, "uniform": 23373111, "epanechnikov": 55945136,
-                    "histogram": 126858990}
+ISSUE_WARP_INSTR = {"fused": 186162180, "uniform": 23372766, "epanechnikov": 58697712,
+                    "histogram": 129411919}
 ISSUE_SOURCE = "profiles/instructions_bench_headline_1024x1024x20.md"
 
 
