@@ -1293,7 +1293,7 @@ __device__ __forceinline__ void integrate_tile(const Field &f, int ty0, int tx0,
         if (!present[i]) {  // F = 1, G = T - F = 1 (semi_cdf)
           nb[i].kind = 0;
           nb[i].lam = 0.f;
-          nb[i].w = nb[i].iw = 0.f;
+          nb[i].w = nb[i].ih = 0.f;
           nb[i].T = 2.f;
           nb[i].off = 0;
           continue;
@@ -1302,7 +1302,7 @@ __device__ __forceinline__ void integrate_tile(const Field &f, int ty0, int tx0,
         nb[i].lam = lo - lo1;
         nb[i].kind = lo == hi ? 2 : 1;
         nb[i].w = hi - lo;
-        nb[i].iw = lo == hi ? 0.f : 1.f / (hi - lo);
+        nb[i].ih = lo == hi ? 0.f : (float)f.B / (hi - lo);
       }
       const PhiloxKeys K(f.seed_lo, f.seed_hi);
       const uint32_t vid = (uint32_t)((long long)gy * f.W + gx);
