@@ -1219,12 +1219,16 @@ __device__ __forceinline__ void semi_sums(const float *tab, int l, float h1, con
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     base[i] = static_cast<uint32_t>(__cvta_generic_to_shared(tab + nb[i].off)) - kTwo23 * (8u * WS);
-    // 1 / w rounded once: B / w times 1 / B and its residual (the product alone
-    // gives 3, 5 and 10 bins a mean error 8 to 20 % larger; the quotient formed
-    // before the loop cost grids of one wave 7 %: 191 x 124 x 40, 4 bins 126 us
-    // against 120); kept as it is where it is 0 or infinite
-    const float a = nb[i].ih * (1.f / Bf), r = fmaf(-nb[i].w, a, 1.f);
-    iw[i] = fabsf(r) < 0.5f ? fmaf(a, r, a) : a;
+    // 1 / w rounded once: B / w times 1 / B (exact where B is a power of two)
+    // and its residual (the product alone gives 3, 5 and 10 bins a mean error 8
+    // to 20 % larger; the quotient formed before the loop cost grids of one wave
+    // 7 %: 191 x 124 x 40, 4 bins 126 us against 120); kept as it is where it is
+    // 0 or infinite
+    iw[i] = nb[i].ih * (1.f / Bf);
+    if constexpr (LOG < 0 && !PM) {
+      const float r = fmaf(-nb[i].w, iw[i], 1.f);
+      if (fabsf(r) < 0.5f) iw[i] = fmaf(iw[i], r, iw[i]);
+    }
   }
   Kahan2 acc;
   auto sample = [&](uint32_t wa, uint32_t wb) {
