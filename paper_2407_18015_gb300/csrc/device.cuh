@@ -609,7 +609,8 @@ struct EpanInv {
 // factor at a time; now the two are equal.  Nodes in pairs, one per half of a
 // float2 (packed FP32 instructions).  1024 x 1024 vertices from parameters:
 // minimum and maximum 50 us, saddle 77 (one factor at a time 56 and 130, single
-// floats 44 and 62); three models of 1024 x 1024 x 20 220 us (224, 218).
+// floats 44 and 62); three models of 1024 x 1024 x 20 220 us (218 with single
+// floats).
 // A factor that starts at the range's end enters pieces of zero width alone,
 // where nothing bounds q: they are 0.
 // NG: the rule, if fewer nodes do (the product is known to have a lower
