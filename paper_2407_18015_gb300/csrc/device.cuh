@@ -1483,7 +1483,8 @@ __device__ __forceinline__ void lds128_cross(float nx, float x1, uint32_t &addr,
 }
 // The same in two 8-byte reads: a 16-byte one wants four adjacent registers,
 // and the packed arithmetic of a walk unrolled twice moves between pairs (1024
-// x 1024 vertices from parameters, 16 bins, both types 263 -> 254 us).
+// x 1024 vertices from parameters, 16 bins, both types 263 -> 254 us, although
+// lanes 16 bytes apart share banks in twos).
 template <unsigned stride>
 __device__ __forceinline__ void lds2x64_cross(float nx, float x1, uint32_t &addr, float4 &v) {
   asm("{\n .reg .pred q;\n setp.le.f32 q, %5, %6;\n"
