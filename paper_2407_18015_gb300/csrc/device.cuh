@@ -1471,12 +1471,20 @@ __device__ __forceinline__ void hist_walk(const float *S0, int coff, int B, floa
 
 // Crossing step of a walker over shared-memory rows: if nx <= x1, read the
 // 16-byte row at addr into v and advance addr by `stride` bytes; else leave
-// both.  One comparison, predicated reads and a predicated add, no branch.  Two
-// 8-byte reads: a 16-byte one wants four adjacent registers, and the packed
-// arithmetic of a walk unrolled twice moves between pairs (1024 x 1024 vertices
-// from parameters, 16 bins, both types 263 -> 254 us, eight neighbours 962 ->
-// 912, although lanes 16 bytes apart share banks in twos).  addr: a
-// shared-state-space address.
+// both.  One comparison, predicated reads and a predicated add, no branch.
+// addr: a shared-state-space address.
+template <unsigned stride>
+__device__ __forceinline__ void lds128_cross(float nx, float x1, uint32_t &addr, float4 &v) {
+  asm("{\n .reg .pred q;\n setp.le.f32 q, %5, %6;\n"
+      " @q ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];\n"
+      " @q add.u32 %4, %4, %7;\n}"
+      : "+f"(v.x), "+f"(v.y), "+f"(v.z), "+f"(v.w), "+r"(addr)
+      : "f"(nx), "f"(x1), "n"(stride));
+}
+// The same in two 8-byte reads: a 16-byte one wants four adjacent registers,
+// and the packed arithmetic of a walk unrolled twice moves between pairs (1024
+// x 1024 vertices from parameters, 16 bins, both types 263 -> 254 us, although
+// lanes 16 bytes apart share banks in twos).
 template <unsigned stride>
 __device__ __forceinline__ void lds2x64_cross(float nx, float x1, uint32_t &addr, float4 &v) {
   asm("{\n .reg .pred q;\n setp.le.f32 q, %5, %6;\n"
@@ -1622,12 +1630,13 @@ __device__ __forceinline__ float fmin5(float a, float b, float c, float d, float
   return r;
 }
 
-// A walker's crossing in a walk of mode MODE.
-template <int RS, int MODE>
+// A walker's crossing in a walk of mode MODE; QUAD: rows read whole.
+template <int RS, int MODE, bool QUAD = false>
 __device__ __forceinline__ void walker_cross(float nx, float x1, HistRowWalker &n) {
   constexpr unsigned stride = (unsigned)(RS * 16);
   if constexpr (MODE == kWalkMin) lds_cross1<stride, 0>(nx, x1, n.addr, n.r.x, n.r.z, n.r.w);
   else if constexpr (MODE == kWalkMax) lds_cross1<stride, 4>(nx, x1, n.addr, n.r.y, n.r.z, n.r.w);
+  else if constexpr (QUAD) lds128_cross<stride>(nx, x1, n.addr, n.r);
   else lds2x64_cross<stride>(nx, x1, n.addr, n.r);
 }
 

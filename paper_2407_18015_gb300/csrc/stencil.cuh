@@ -379,60 +379,58 @@ __device__ __forceinline__ void hist_walk_k(const float *tab, long long crow, in
   pmax = fmaxf(acc.y, 0.f);
 }
 
-// Mean over a piece of the product of K = 6 or 8 linear factors given by their
-// left and right values: pairs of factors are quadratics (b0, b1, b2) in the
-// Bernstein basis (b1 doubled), two pairs a quartic c_0..c_4 (with the
-// basis' binomials), and with d the third pair or the other quartic
-//   mean = sum_kl c_k d_l / ((K + 1) C(K, k + l)).
-// Every term is a product of non-negative end values: 41 and 64 operations (53
-// and 79 for the binomial expansion factor by factor).  Over fitted masses of 5
-// to 16 bins the walk's mean error against 64 bits is 0.99 to 1.04 times that
-// of the expansion; with the moments about the middle, as many operations, it
-// was 0.93 to 1.11 times.
+// Mean over [-1, 1] of the product of K = 6 or 8 linear factors m_i - D_i t,
+// from their middle values and half falls: pairs of factors are quadratics p -
+// b t + e t^2, two pairs a quartic, and the mean of a product of polynomials
+// is the sum of its even coefficients over 1, 3, 5, ... .  Every term is a
+// product of non-negative numbers.  O: the arithmetic of one or both types
+// (HistWalkOps); with both, the odd coefficients of F carry the opposite
+// sign, which drops out (they meet in pairs).
 template <int K, typename O, typename V>
-__device__ __forceinline__ V bern_mean_pairs_k(const V *L, const V *R) {
+__device__ __forceinline__ V linear_mean_k(const V *m, const V *D) {
   static_assert(K == 6 || K == 8, "three or four pairs");
-  constexpr int P = K / 2, ND = K == 6 ? 3 : 5;
-  V b[P][3];
+  constexpr int P = K / 2;
+  V p[P], b[P], e[P];
 #pragma unroll
   for (int j = 0; j < P; ++j) {
-    const V *l = L + 2 * j, *r = R + 2 * j;
-    b[j][0] = O::mul(l[0], l[1]);
-    b[j][1] = O::fma(l[0], r[1], O::mul(r[0], l[1]));
-    b[j][2] = O::mul(r[0], r[1]);
+    p[j] = O::mul(m[2 * j], m[2 * j + 1]);
+    e[j] = O::mul(D[2 * j], D[2 * j + 1]);
+    b[j] = O::fma(m[2 * j], D[2 * j + 1], O::mul(m[2 * j + 1], D[2 * j]));
   }
-  auto quartic = [&](const V *x, const V *y, V *q) {
-    q[0] = O::mul(x[0], y[0]);
-    q[1] = O::fma(x[0], y[1], O::mul(x[1], y[0]));
-    q[2] = O::fma(x[0], y[2], O::fma(x[1], y[1], O::mul(x[2], y[0])));
-    q[3] = O::fma(x[1], y[2], O::mul(x[2], y[1]));
-    q[4] = O::mul(x[2], y[2]);
+  const V c3 = O::all(1.f / 3.f), c5 = O::all(0.2f), c7 = O::all(1.f / 7.f);
+  // the quartic of two pairs: coefficients of 1, -t, t^2, -t^3, t^4
+  auto quartic = [&](int i, int j, V *q) {
+    q[0] = O::mul(p[i], p[j]);
+    q[1] = O::fma(p[i], b[j], O::mul(b[i], p[j]));
+    q[2] = O::fma(p[i], e[j], O::fma(b[i], b[j], O::mul(e[i], p[j])));
+    q[3] = O::fma(b[i], e[j], O::mul(e[i], b[j]));
+    q[4] = O::mul(e[i], e[j]);
   };
-  V c[5], d[ND];
-  quartic(b[0], b[1], c);
+  V q[5];
+  quartic(0, 1, q);
   if constexpr (K == 6) {
-#pragma unroll
-    for (int l = 0; l < 3; ++l) d[l] = b[2][l];
+    const V u0 = O::fma(e[2], c3, p[2]);
+    const V u2 = O::fma(p[2], c3, O::mul(e[2], c5));
+    const V u4 = O::fma(p[2], c5, O::mul(e[2], c7));
+    const V v = O::fma(q[3], c5, O::mul(q[1], c3));
+    return O::fma(q[0], u0, O::fma(q[2], u2, O::fma(q[4], u4, O::mul(v, b[2]))));
   } else {
-    quartic(b[2], b[3], d);
+    V r[5];
+    quartic(2, 3, r);
+    const V c9 = O::all(1.f / 9.f);
+    const V u0 = O::fma(r[2], c3, O::fma(r[4], c5, r[0]));
+    const V u2 = O::fma(r[0], c3, O::fma(r[2], c5, O::mul(r[4], c7)));
+    const V u4 = O::fma(r[0], c5, O::fma(r[2], c7, O::mul(r[4], c9)));
+    const V v1 = O::fma(r[1], c3, O::mul(r[3], c5));
+    const V v3 = O::fma(r[1], c5, O::mul(r[3], c7));
+    return O::fma(q[0], u0,
+                  O::fma(q[2], u2, O::fma(q[4], u4, O::fma(q[1], v1, O::mul(q[3], v3)))));
   }
-  V s = c[0];
-#pragma unroll
-  for (int k = 0; k < 5; ++k) {
-    V t = O::mul(d[0], O::all(bern_w(K, k)));
-#pragma unroll
-    for (int l = 1; l < ND; ++l) t = O::fma(d[l], O::all(bern_w(K, k + l)), t);
-    s = k == 0 ? O::mul(c[0], t) : O::fma(c[k], t, s);
-  }
-  return s;
 }
 
 // hist_walk_pieces with K neighbours: the same rows, walkers and steps (every
-// lane runs the same instructions, the crossings predicated; two pieces per
-// turn, the second clamped to the walk's end); MODE kWalkBoth, kWalkMin or
-// kWalkMax.  1024 x 1024 vertices from parameters, eight neighbours, 8 bins:
-// both types 490 us, one 352 (one piece per turn 534 and 376; with the moments
-// about the middle and 16-byte reads 482 and 364).
+// lane runs the same instructions, the crossings predicated); MODE kWalkBoth,
+// kWalkMin or kWalkMax.
 template <int K, int RS, int MODE>
 __device__ __forceinline__ void hist_walk_rows_k(const float4 *crow, int B, float W1,
                                                  HistRowWalker *nw, float &pmin, float &pmax) {
@@ -450,7 +448,9 @@ __device__ __forceinline__ void hist_walk_rows_k(const float4 *crow, int B, floa
   }
   V acc = O::all(0.f);
   float x0 = 0.f;
-  auto piece = [&](bool clamp) {
+  const int max_steps = (K + 1) * (B + 1) + 4;
+#pragma unroll 1
+  for (int step = 0; step < max_steps && x0 < W1; ++step) {
     float e[K];
     float x1 = dc.y;
 #pragma unroll
@@ -458,35 +458,30 @@ __device__ __forceinline__ void hist_walk_rows_k(const float4 *crow, int B, floa
       e[i] = nw[i].nx();
       x1 = fminf(x1, e[i]);
     }
-    if (clamp) x1 = fminf(x1, W1);
-    const float d = x1 - x0;
-    V L[K], R[K];  // left and right values; the walkers move to x1
+    const float d = x1 - x0, hd = 0.5f * d;
+    V m[K], D[K];
 #pragma unroll
     for (int i = 0; i < K; ++i) {
       float4 &r = nw[i].r;
       if constexpr (O::two) {
-        L[i] = make_float2(r.x, r.y);
-        R[i] = __ffma2_rn(make_float2(r.z, r.z), make_float2(-d, d), L[i]);
-        r.x = R[i].x;
-        r.y = R[i].y;
+        const float2 zz = make_float2(r.z, r.z), l = make_float2(r.x, r.y);
+        D[i] = __fmul2_rn(zz, make_float2(hd, hd));
+        m[i] = __ffma2_rn(zz, make_float2(-hd, hd), l);
+        const float2 v = __ffma2_rn(zz, make_float2(-d, d), l);
+        r.x = v.x;
+        r.y = v.y;
       } else {
         float &l = MODE == kWalkMin ? r.x : r.y;
-        L[i] = l;
+        D[i] = __fmul_rn(r.z, hd);
+        m[i] = __fmaf_rn(r.z, MODE == kWalkMin ? -hd : hd, l);
         l = __fmaf_rn(r.z, MODE == kWalkMin ? -d : d, l);
-        R[i] = l;
       }
     }
-    acc = O::fma(O::all(__fmul_rn(d, dc.x)), bern_mean_pairs_k<K, O>(L, R), acc);
+    acc = O::fma(O::all(__fmul_rn(d, dc.x)), linear_mean_k<K, O>(m, D), acc);
 #pragma unroll
-    for (int i = 0; i < K; ++i) walker_cross<RS, MODE>(e[i], x1, nw[i]);
+    for (int i = 0; i < K; ++i) walker_cross<RS, MODE, true>(e[i], x1, nw[i]);
     lds64_cross<(unsigned)(RS * 16)>(dc.y, x1, addr_c, dc);
     x0 = x1;
-  };
-  const int max_steps = (K + 1) * (B + 1) + 4;
-#pragma unroll 1
-  for (int step = 0; step < max_steps && x0 < W1; step += 2) {
-    piece(false);
-    piece(true);
   }
   if constexpr (O::two) {
     pmin = fmaxf(acc.x, 0.f);
